@@ -79,3 +79,16 @@ def test_special_values(helper):
     x = np.array(vals + [-v for v in vals])
     o, r = run(helper, x)
     assert_bitwise(o, r, x)
+
+
+@pytest.mark.parametrize("low", ["zero", "ones", "random"])
+def test_every_seed(helper, low):
+    """All 2^23 leading significands (one binary32 seed each), with the low
+    29 bits at both ends of the interval that shares the seed and inside it."""
+    g = np.random.Generator(np.random.Philox(33))
+    top = np.arange(1 << 23, dtype=np.uint64) << np.uint64(29)
+    tail = {"zero": np.uint64(0), "ones": np.uint64((1 << 29) - 1),
+            "random": g.integers(0, 1 << 29, size=1 << 23, dtype=np.uint64)}[low]
+    x = (np.uint64(1023 << 52) | top | tail).view(np.float64)
+    o, r = run(helper, x)
+    assert_bitwise(o, r, x)
