@@ -62,7 +62,7 @@ SPILL_ALLOW = [
     # store phases on the stack (the same with a higher register limit);
     # the refinement warp kernel at 64 registers (8 blocks per SM, measured
     # faster than 7 blocks without the spill)
-    (r"k_smem_group|k_smem_ragged|k_smem_ir|k_ragged_persist", 32, 32),
+    (r"k_smem_group|k_smem_ragged|k_smem_ir|k_ragged_persist", 48, 48),
 ]
 
 # (n, lanes per system) kernel families compiled into the library.

@@ -74,19 +74,47 @@ int default_ragged_id(int n)
     return variant_id(n <= 26 ? 16 : 32, 1);
 }
 
-// Default gesv/getrf variant id per n before any autotuning: the variant
-// tl_autotune found fastest at each n on a GB300 (interleaved batches of
-// about 1.6 GFLOP per n).  One thread per system in registers up to n = 9,
-// then the two-step element walk in shared memory with 2, 4, 8, 16 and 32
-// lanes per system (16 up to n = 30, 32 at n = 31, 32).
-int default_lanes(int n)
+// Default variant id of an operation before any autotuning: one thread per
+// system in registers up to n = 9, then the two-step element walk in shared
+// memory.  The lines are where the next lane count becomes faster, measured
+// on a GB300 on batches of about 1.6 GFLOP (TFLOP/s on both sides):
+// interleaved gesv n = 10: 2 lanes 0.89, 4 lanes 0.80; n = 11: 0.85, 0.86;
+// n = 17: 4 lanes 0.89, 8 lanes 0.87; n = 18: 0.85, 0.88; n = 24: 8 lanes
+// 0.85, 16 lanes 0.81; n = 25: 0.82, 0.86; 32 lanes never (n = 32: 0.82
+// against 0.87).  Per system 8 lanes already win at n = 17 (0.92 against
+// 0.90) and up to n = 26 (0.90, 0.90).  With the factors stored the next lane
+// count wins earlier, and 32 lanes from n = 27 on (interleaved, 0.745 against
+// 0.707) or n = 31 (per system, 0.868 against 0.860).
+int default_lanes(int n, int layout, int op)
 {
+    const bool inter = layout == TL_LAYOUT_INTERLEAVED;
     if (n <= 9) return variant_id(1, 0);
-    if (n <= 11) return variant_id(2, 2);
-    if (n <= 15) return variant_id(4, 2);
-    if (n <= 23) return variant_id(8, 2);
-    if (n <= 30) return variant_id(16, 1);
-    return variant_id(32, 1);
+    if (op == kOpGesvLU || op == kOpGetrf) {
+        if (n <= 10) return variant_id(2, 2);
+        if (n <= 14) return variant_id(4, 2);
+        if (n <= (inter ? 24 : 22)) return variant_id(8, 2);
+        return n <= (inter ? 26 : 30) ? variant_id(16, 1) : variant_id(32, 1);
+    }
+    if (n <= 10) return variant_id(2, 2);
+    if (n <= (inter ? 17 : 16)) return variant_id(4, 2);
+    return n <= (inter ? 24 : 26) ? variant_id(8, 2) : variant_id(16, 1);
+}
+
+// Default block size of the shared-memory kernels (0: the occupancy and wave
+// heuristic, for the register kernels).  Per system every warp copies its own
+// systems, so one-warp blocks are best (nothing waits at the block barrier:
+// n = 21, 8 lanes 0.94 TFLOP/s, 0.90 with 64 threads, 0.88 with 128).
+// Interleaved, a block of b threads reads 8 b / lanes consecutive bytes of
+// each entry: 64 threads for up to 8 lanes (n = 19: 0.87, with 128 threads
+// 0.85), 128 above (n = 30: 0.89, with 64 0.86); one warp is enough for 2
+// and 4 lanes (n = 13: 0.89, 64 threads 0.88), also when the batch would
+// otherwise leave SMs without a block.
+int default_block(tl_handle *h, const Variant *v, int layout, int64_t batch)
+{
+    if (v->kind == 0) return 0;
+    if (layout == TL_LAYOUT_PER_SYSTEM || v->lanes <= 4) return 32;
+    const int block = v->lanes <= 8 ? 64 : 128;
+    return batch * v->lanes < static_cast<int64_t>(block) * h->sm_count ? 32 : block;
 }
 
 // Variant by id (lanes + 100 * kind); falls back to the register kernel of
@@ -215,9 +243,9 @@ tl_status launch_variant(tl_handle *h, const Variant *v, int n, int block, Solve
 tl_status launch_op(tl_handle *h, int n, int layout, int op, SolveArgs &args, cudaStream_t stream)
 {
     const Choice &c = h->choice[n][layout][op];
-    const Variant *v = find_variant(n, layout, op, c.lanes ? c.lanes : default_lanes(n));
+    const Variant *v = find_variant(n, layout, op, c.lanes ? c.lanes : default_lanes(n, layout, op));
     if (!v) return TL_ERR_UNSUPPORTED;
-    return launch_variant(h, v, n, c.block, args, stream);
+    return launch_variant(h, v, n, c.lanes ? c.block : default_block(h, v, layout, args.batch), args, stream);
 }
 
 static bool misaligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) != 0; }

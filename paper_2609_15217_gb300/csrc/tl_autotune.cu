@@ -135,7 +135,7 @@ extern "C" tl_status tl_dispatch_get(tl_handle *h, int n, tl_layout layout, int 
     if (layout != TL_LAYOUT_PER_SYSTEM && layout != TL_LAYOUT_INTERLEAVED) return fail_arg(h, 3);
     if (!variant) return fail_arg(h, 4);
     const Choice &c = h->choice[n][layout][kOpGesv];
-    const Variant *v = find_variant(n, layout, kOpGesv, c.lanes ? c.lanes : default_lanes(n));
+    const Variant *v = find_variant(n, layout, kOpGesv, c.lanes ? c.lanes : default_lanes(n, layout, kOpGesv));
     *variant = v ? variant_id(v->lanes, v->kind) : 0;
     if (block) *block = c.block;
     return TL_OK;

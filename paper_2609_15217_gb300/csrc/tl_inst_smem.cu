@@ -7,20 +7,17 @@
 namespace tl {
 namespace {
 
-// ASYNC: cp.async loads into shared memory (the 2..8-lane kernels, 20-40%
-// faster than staged loads); 16 and 32 lanes per system measured 4-8% faster
-// with register-staged streaming loads.
-template <int T, int L, bool WALK = (T >= 16), bool ASYNC = (T < 16)>
+template <int T, int L, bool WALK = (T >= 16)>
 void reg_smem()
 {
     constexpr int kind = (WALK && T < 16) ? 2 : 1;
     for (int n = 2; n <= TL_MAX_N; ++n) {
         register_variant(n, L, kOpGesv, T,
-                         reinterpret_cast<const void *>(&k_smem_group<T, L, kGesv, false, WALK, ASYNC>), kind);
+                         reinterpret_cast<const void *>(&k_smem_group<T, L, kGesv, false, WALK>), kind);
         register_variant(n, L, kOpGesvLU, T,
-                         reinterpret_cast<const void *>(&k_smem_group<T, L, kGesv, true, WALK, ASYNC>), kind);
+                         reinterpret_cast<const void *>(&k_smem_group<T, L, kGesv, true, WALK>), kind);
         register_variant(n, L, kOpGetrf, T,
-                         reinterpret_cast<const void *>(&k_smem_group<T, L, kGetrf, true, WALK, ASYNC>), kind);
+                         reinterpret_cast<const void *>(&k_smem_group<T, L, kGetrf, true, WALK>), kind);
     }
 }
 

@@ -106,7 +106,8 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) k_newton_tanh_smem(Newton
         const bool need = have && st < 0;
         __syncwarp();
         if (__any_sync(0xffffffffu, need)) {
-            const int info = smem_lupp2<T, true, false>(M, n, RS, t, 0, 0.0);
+            unsigned worst;  // a non-finite Jacobian shows in the next residual
+            const int info = smem_lupp2<T, true, false>(M, n, RS, t, 0, 0.0, worst);
             if (need) {
                 if (info != 0) {
                     st = TL_NEWTON_SINGULAR;

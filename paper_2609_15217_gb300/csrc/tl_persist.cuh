@@ -95,16 +95,11 @@ __device__ __forceinline__ void persist_item(const RaggedArgs &r, int n, int64_t
     cp_async_wait_all();
     __syncwarp();
     double *M = W + q * per;
-    // a non-finite entry anywhere in the group's system
-    int badv = 0;
-    if (first + q < count) {
-        for (int e = t; e < nn; e += T) {
-            const int j = div20(e, m20);
-            badv |= dev::is_nonfinite(M[(e - j * n) * RS + j]) ? 1 : 0;
-        }
-    }
-    const bool bad = group_any_int<T>(badv) != 0;
-    int info = smem_lupp2<T, true, false>(M, n, RS, t, 0, 0.0);
+    unsigned worst = 0;
+    int info = smem_lupp2<T, true, false>(M, n, RS, t, 0, 0.0, worst);
+    const int64_t ao = __shfl_sync(0xffffffffu, my_a, q);
+    const bool bad = smem_bad_input<T>(first + q < count && worst >= 0x7ff00000u,
+                                       first + q < count ? r.A + ao : nullptr, nn, t);
     if (bad) info = -1;
     const int64_t s = __shfl_sync(0xffffffffu, my_s, q);
     const int64_t xo = __shfl_sync(0xffffffffu, my_b, q);

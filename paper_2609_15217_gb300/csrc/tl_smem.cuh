@@ -13,10 +13,9 @@
 //   * smem_lupp: one step per pass on a TR x TC tile of lanes (lane (tr, tc)
 //     keeps its columns of the pivot row in registers and walks its rows)
 //     or an element walk; kept for the lane-tile variants.
-// The kernels: k_smem_group (fixed-size batches, both layouts; loads into
-// shared memory by cp.async for 2..8 lanes and by register-staged streaming
-// loads for 16 and 32 lanes, the faster choice measured for each) and
-// k_smem_ragged (one size of a ragged batch, the per-size mode).
+// The kernels: k_smem_group (fixed-size batches, both layouts, loads into
+// shared memory by cp.async) and k_smem_ragged (one size of a ragged batch,
+// the per-size mode).
 //
 // Arithmetic is the same as the register solvers of tinylu_device.cuh (negated
 // multipliers a_ik * (-RN(1/a_kk)), one FMA per update in increasing k, the
@@ -55,7 +54,7 @@ __host__ __device__ constexpr int smem_piv_offset(int n) { return n * smem_row_s
 __host__ __device__ constexpr int smem_sys_doubles(int n, int T = 16)
 {
     const int base = smem_piv_offset(n) + (n + 1) / 2;
-    const int want = (T < 16) ? T : 0;
+    const int want = T < 16 ? T : T / 8;
     return base + ((want - base % 16) % 16 + 16) % 16;
 }
 __host__ __device__ constexpr size_t smem_sys_bytes(int n, int T = 16)
@@ -254,24 +253,36 @@ __device__ __forceinline__ int smem_lupp(double *M, int n, int RS, int t, int ti
 // Element-walk elimination with the trailing update of two steps per pass.
 //
 // Same result as smem_lupp<T, SOLVE, true> bit for bit (every element still
-// receives fma(-l_ik, u_kj, a_ij) in increasing k with the same operands),
-// organized to issue fewer instructions per FMA, which measured as the
-// bottleneck of the one-step walk (about 50 warp instructions per FP64
-// instruction, the FP64 pipe 67-77% busy):
+// receives fma(-l_ik, u_kj, a_ij) in increasing k with the same operands).
+// Bound by the FP64 pipe (64 clocks of a sub-partition per warp instruction,
+// full or not) and, in between, by the latency of each step's serial part:
+// the pivot search, the reciprocal, the interchange and the multipliers took
+// 43,000 of the 73,000 clocks that a warp alone on an SM needed for four
+// systems of n = 19, against 24,600 of FP64 instructions, too much for the
+// three or four warps per sub-partition to hide.  So:
 //   * steps k and k+1 are paired: after the pivot of step k (search, row
 //     interchange, multipliers, column k+1 updated in the same pass), the
-//     pivot of step k+1 is found, row k+1 receives its step-k update and
-//     column k+1 its multipliers; then one walk over the block below and to
-//     the right of (k+1, k+1) applies both steps' updates to each element
-//     (one load, two FMAs in order, one store).  Rows interchanged at step
-//     k+1 still carry their pending step-k update and their own -l_ik, so
-//     the interchange covers column k as well.
-//   * with a full warp per system the pivot search is three warp reductions
-//     (redux.sync) on the high and low words of the magnitude and on the row;
+//     pivot of step k+1 is found among the values that pass just formed, the
+//     row that becomes row k+1 receives its step-k update during its
+//     interchange and column k+1 its multipliers; then one walk over the
+//     block below and to the right of (k+1, k+1) applies both steps' updates
+//     to each element (one load, two FMAs in order, one store).  Rows
+//     interchanged at step k+1 still carry their pending step-k update and
+//     their own -l_ik, so the interchange covers column k as well;
+//   * every serial pass loads what it needs before its first arithmetic or
+//     store (PivotScan, smem_swap, smem_multipliers), and passes end with
+//     branches the whole warp takes: an FP64 instruction without an active
+//     lane costs as much as a full one;
 //   * element walk indices come from a multiply-shift instead of run-time
 //     divisions;
 //   * the back substitution keeps y in registers (lane t holds rows
-//     t, t+T, ...) and broadcasts each x_i with a shuffle.
+//     t, t+T, ...) and broadcasts each x_i with a shuffle;
+//   * whether A holds a non-finite entry is learned on the way (worst).
+// Measured against the first form of this walk (search from shared memory by
+// warp reductions, one entry at a time in every pass, a scan of A for
+// non-finite entries): n = 19 per system, 313,111 systems, 0.80 -> 0.93
+// TFLOP/s; n = 13 interleaved, 932,944 systems, 0.84 -> 0.89; n = 30 per
+// system, 82,712 systems, 0.89 -> 0.94.
 // KEEPL: interchange whole rows, L part included (getrf output); without it
 // only the columns the remaining elimination reads are interchanged.
 // ---------------------------------------------------------------------------
@@ -292,151 +303,245 @@ __device__ __forceinline__ int div_small(int x, int c)
     return c == 1 ? x : static_cast<int>((static_cast<unsigned>(x) * kDivMagic.m[c]) >> 16);
 }
 
-// First maximum of |M[i*RS + k]| over candidate rows i in [lo, hi) of the
-// group; every lane of the group receives the pivot row and value.  lim is
-// the size of the system's block (checked builds, see tl_bounds.cuh).
+// First maximum of |M[i*RS + k]| over rows i in [lo, hi) of the group's
+// system: a butterfly over (magnitude, row).  Every lane of the warp together.
+// The rare second stage of the pivot search, out of line.
 template <int T>
-__device__ __forceinline__ void smem_pivot_search(const double *M, int RS, int k, int lo, int hi, int t, int lim,
-                                                  double &cv, int &cpos)
+static __device__ __noinline__ int smem_pivot_exact(const double *M, int RS, int k, int lo, int hi, int t, int lim)
 {
-    if constexpr (T == 32) {
-        // one candidate per lane (n <= 32): reduce the high word, the low
-        // word among the lanes holding the largest high word, then the row
-        const int i = lo + t;
-        const bool cand = i < hi;
-        const unsigned long long m = cand ? dev::mag_bits(TL_SM(M, i * RS + k, lim)) : 0ULL;
-        const unsigned mh = static_cast<unsigned>(m >> 32), ml = static_cast<unsigned>(m);
-        const unsigned maxh = __reduce_max_sync(0xffffffffu, cand ? mh : 0u);
-        const bool c2 = cand && mh == maxh;
-        const unsigned maxl = __reduce_max_sync(0xffffffffu, c2 ? ml : 0u);
-        const bool c3 = c2 && ml == maxl;
-        cpos = static_cast<int>(__reduce_min_sync(0xffffffffu, c3 ? static_cast<unsigned>(i) : 0xffffffffu));
-        cv = TL_SM(M, cpos * RS + k, lim);
-    } else if constexpr (T == 16 || T == 8) {
-        // 32 / T systems per warp: each lane's first maximum over its rows,
-        // then the same three reductions once per group (the lanes of the
-        // other groups contribute the neutral value).  Measured against the
-        // shuffle butterfly below: 2.4-4.4% faster at n = 24..28 with 16
-        // lanes, 0.4-1.6% at n = 18..21 with 8
-        constexpr int G = 32 / T;
-        unsigned long long best = 0;
-        int row = hi;
-        for (int i = lo + t; i < hi; i += T) {
-            const unsigned long long m = dev::mag_bits(TL_SM(M, i * RS + k, lim));
-            if (row == hi || m > best) {
-                best = m;
-                row = i;
+    unsigned long long best = 0;
+    int row = hi;
+    for (int i = lo + t; i < hi; i += T) {
+        const unsigned long long m = dev::mag_bits(TL_SM(M, i * RS + k, lim));
+        if (row == hi || m > best) {
+            best = m;
+            row = i;
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int off = T / 2; off >= 1; off >>= 1) {
+        const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, off);
+        const int orow = __shfl_xor_sync(0xffffffffu, row, off);
+        const bool take = (orow < hi) && (row >= hi || ob > best || (ob == best && orow < row));
+        best = take ? ob : best;
+        row = take ? orow : row;
+    }
+    return row;
+}
+
+// Pivot search of one column.  Each lane proposes its candidates (add), then
+// the group agrees (finish) on the largest high word of |a_ik|: log2(T)
+// 32-bit shuffles (one warp reduction for T = 32), one vote, one shuffle of
+// the winner.  Two candidates that share the largest high word (1e-5 of the
+// columns of random systems, most columns of small integers) take the exact
+// search on the whole magnitude.  On one warp per SM, n = 19 with 8 lanes:
+// 470 clocks per search, 670 with a warp reduction of the high word, the low
+// word and the row for each group.
+struct PivotScan {
+    unsigned best;  // high word of the largest magnitude + 1, 0 without a candidate
+    double v;
+    int row;
+    bool tie;
+    __device__ __forceinline__ void clear()
+    {
+        best = 0;
+        v = 0.0;
+        row = 0;
+        tie = false;
+    }
+    __device__ __forceinline__ void add(double a, int i, bool in)
+    {
+        const unsigned key = in ? static_cast<unsigned>(dev::mag_bits(a) >> 32) + 1u : 0u;
+        const bool gt = key > best;
+        tie = gt ? false : (tie || (in && key == best));
+        best = gt ? key : best;
+        v = dev::sel(gt, a, v);
+        row = gt ? i : row;
+    }
+    template <int T>
+    __device__ __forceinline__ void finish(const double *M, int RS, int k, int lo, int hi, int t, int lim, double &cv,
+                                           int &p) const
+    {
+        constexpr unsigned kMask = T == 32 ? 0xffffffffu : (1u << (T & 31)) - 1u;
+        const int lane0 = (static_cast<int>(threadIdx.x) & 31) - t;
+        unsigned m = best;
+        if constexpr (T == 32) {
+            m = __reduce_max_sync(0xffffffffu, m);
+        } else {
+#pragma unroll
+            for (int off = T / 2; off >= 1; off >>= 1) {
+                const unsigned o = __shfl_xor_sync(0xffffffffu, m, off);
+                m = o > m ? o : m;
             }
         }
-        const int grp = static_cast<int>(threadIdx.x & 31u) / T;
-        const bool cand = row < hi;
-        const unsigned mh = static_cast<unsigned>(best >> 32), ml = static_cast<unsigned>(best);
-        unsigned maxh = 0;
+        const bool mine = best == m;
+        const unsigned who = (__ballot_sync(0xffffffffu, mine) >> lane0) & kMask;
+        const bool ambiguous = (who & (who - 1u)) != 0u || (mine && tie);
+        if (__any_sync(0xffffffffu, ambiguous)) {
+            p = smem_pivot_exact<T>(M, RS, k, lo, hi, t, lim);
+            cv = TL_SM(M, p * RS + k, lim);
+            __syncwarp();  // before the interchange writes the column
+        } else {
+            const int w = lane0 + __ffs(static_cast<int>(who)) - 1;
+            p = __shfl_sync(0xffffffffu, row, w);
+            cv = __shfl_sync(0xffffffffu, v, w);
+        }
+    }
+};
+
+// Rows (multipliers) of one lane per pass: every row of its share in one
+// pass from 8 lanes on.
+template <int T>
+struct RowChunk {
+    static constexpr int U = TL_MAX_N / T < 4 ? TL_MAX_N / T : 4;
+};
+
+// Candidates of column k in rows [lo, hi) from shared memory.
+template <int T>
+__device__ __forceinline__ void smem_scan(const double *M, int RS, int k, int lo, int hi, int t, int lim, PivotScan &sc)
+{
+    constexpr int U = RowChunk<T>::U;
+    sc.clear();
+#pragma unroll 1
+    for (int ib = lo; ib < hi; ib += U * T) {
+        double v[U];
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const unsigned v = __reduce_max_sync(0xffffffffu, grp == g && cand ? mh : 0u);
-            maxh = grp == g ? v : maxh;
+        for (int c = 0; c < U; ++c) {
+            const int i = ib + t + c * T;
+            v[c] = i < hi ? TL_SM(M, i * RS + k, lim) : 0.0;
         }
-        const bool c2 = cand && mh == maxh;
-        unsigned maxl = 0;
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const unsigned v = __reduce_max_sync(0xffffffffu, grp == g && c2 ? ml : 0u);
-            maxl = grp == g ? v : maxl;
-        }
-        const bool c3 = c2 && ml == maxl;
-        unsigned rmin = 0;
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const unsigned v =
-                __reduce_min_sync(0xffffffffu, grp == g && c3 ? static_cast<unsigned>(row) : 0xffffffffu);
-            rmin = grp == g ? v : rmin;
-        }
-        cpos = static_cast<int>(rmin);
-        cv = TL_SM(M, cpos * RS + k, lim);
-    } else {
-        unsigned long long best = 0;
-        int row = hi;
-        for (int i = lo + t; i < hi; i += T) {
-            const unsigned long long m = dev::mag_bits(TL_SM(M, i * RS + k, lim));
-            if (row == hi || m > best) {
-                best = m;
-                row = i;
-            }
-        }
-        // butterfly over the T lanes of the group: largest magnitude, ties
-        // (and lanes without a candidate) to the smallest row
-#pragma unroll
-        for (int off = T / 2; off >= 1; off >>= 1) {
-            const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, off);
-            const int orow = __shfl_xor_sync(0xffffffffu, row, off);
-            const bool take = (orow < hi) && (row >= hi || ob > best || (ob == best && orow < row));
-            best = take ? ob : best;
-            row = take ? orow : row;
-        }
-        cpos = row;
-        cv = TL_SM(M, row * RS + k, lim);
+        for (int c = 0; c < U; ++c) sc.add(v[c], ib + t + c * T, ib + t + c * T < hi);
+        if (U * T >= TL_MAX_N) break;
     }
 }
 
-// Pivot of step k: search (whole column, or the tile-local rule), record
-// pivot and info, interchange rows k and p over columns [jlo, wcols).
-template <int T>
-__device__ __forceinline__ void smem_pivot_step(double *M, int n, int RS, int k, int t, int lim, int jlo, int wcols,
-                                                int tile, double threshold, int *piv, double &cv, int &info)
+// Rows the pivot of step k is sought in first (the whole column, or with
+// tile-local pivoting the diagonal tile).
+__device__ __forceinline__ int smem_pivot_limit(int n, int k, int tile)
 {
-    int hi = n;
-    if (tile > 0 && tile < n) hi = min(n, (k / tile + 1) * tile);
-    int p;
-    smem_pivot_search<T>(M, RS, k, k, hi, t, lim, cv, p);
+    return tile > 0 && tile < n ? min(n, (k / tile + 1) * tile) : n;
+}
+
+// The pivot of step k from the group's candidates in rows [k, hi); with
+// tile-local pivoting a best magnitude below the threshold (in some group
+// of the warp) takes the first maximum over the whole column instead.
+template <int T>
+__device__ __forceinline__ void smem_pivot(const double *M, int n, int RS, int k, int hi, int t, int lim,
+                                           double threshold, const PivotScan &sc, int *piv, double &cv, int &p, int &info)
+{
+    sc.finish<T>(M, RS, k, k, hi, t, lim, cv, p);
     if (hi < n && __any_sync(0xffffffffu, dev::mag_bits(cv) < dev::mag_bits(threshold))) {
-        // tile-local pivoting: the in-tile best is below the threshold (in
-        // some group of the warp): the first maximum over the whole column
-        double cv2;
-        int p2;
-        smem_pivot_search<T>(M, RS, k, k, n, t, lim, cv2, p2);
-        const bool below = dev::mag_bits(cv) < dev::mag_bits(threshold);
-        cv = below ? cv2 : cv;
-        p = below ? p2 : p;
+        const int p2 = smem_pivot_exact<T>(M, RS, k, k, n, t, lim);
+        if (dev::mag_bits(cv) < dev::mag_bits(threshold)) {
+            p = p2;
+            cv = TL_SM(M, p2 * RS + k, lim);
+        }
+        __syncwarp();
     }
     if (dev::mag_bits(cv) == 0ULL && info == 0) info = k + 1;
     if (t == 0) TL_SM(piv, k, n) = p;
-    if (p != k) {
-        for (int j = jlo + t; j < wcols; j += T) {
-            const double tmp = TL_SM(M, k * RS + j, lim);
-            TL_SM(M, k * RS + j, lim) = TL_SM(M, p * RS + j, lim);
-            TL_SM(M, p * RS + j, lim) = tmp;
-        }
-    }
 }
 
-// Negated multipliers of column k below row k (quotient for a pivot below
-// DBL_MIN, a sign flip for a zero column); with UPD the same lane also
-// applies step k to the entry of column k+1 of its row.
-template <int T, bool UPD>
-__device__ __forceinline__ void smem_multipliers(double *M, int n, int RS, int k, int t, int lim, double cv,
-                                                 double nr, bool zero, bool small)
+// Interchange rows k and p over the columns [jlo, wcols), the entries of a
+// pass loaded before its first store.  PEND (the second step of a pair, row
+// k = kp + 1): columns from kp + 2 on of the row that becomes row k receive
+// step kp on the way (l: its negated multiplier, upd: unless step kp's pivot
+// was zero).  worst collects the largest high word of |.| of the new row k.
+template <int T, bool PEND>
+__device__ __forceinline__ void smem_swap(double *M, int n, int RS, int k, int p, int t, int lim, int jlo, int wcols,
+                                          double l, bool upd, unsigned &worst)
 {
-    const double ukk1 = UPD ? TL_SM(M, k * RS + k + 1, lim) : 0.0;
-    if (!__any_sync(0xffffffffu, small)) {
-        for (int i = k + 1 + t; i < n; i += T) {
-            const double l = zero ? dev::neg(TL_SM(M, i * RS + k, lim)) : __dmul_rn(TL_SM(M, i * RS + k, lim), nr);
-            TL_SM(M, i * RS + k, lim) = l;
-            if (UPD && !zero) TL_SM(M, i * RS + k + 1, lim) = __fma_rn(l, ukk1, TL_SM(M, i * RS + k + 1, lim));
+    constexpr int U = T == 32 ? 2 : T == 16 ? 3 : T == 8 ? 5 : 4;
+    const int first = PEND ? k + 1 : jlo;
+    const int rk = k * RS, rp = p * RS, ru = (k - 1) * RS;
+    if (PEND) {  // the columns without an update
+        for (int j = jlo + t; j < first; j += T) {
+            const double vk = TL_SM(M, rk + j, lim);
+            TL_SM(M, rk + j, lim) = TL_SM(M, rp + j, lim);
+            TL_SM(M, rp + j, lim) = vk;
         }
-    } else {
-        const double ncv = dev::neg(cv);
-        for (int i = k + 1 + t; i < n; i += T) {
-            const double a = TL_SM(M, i * RS + k, lim);
-            const double l = zero ? dev::neg(a) : (small ? __ddiv_rn(a, ncv) : __dmul_rn(a, nr));
-            TL_SM(M, i * RS + k, lim) = l;
-            if (UPD && !zero) TL_SM(M, i * RS + k + 1, lim) = __fma_rn(l, ukk1, TL_SM(M, i * RS + k + 1, lim));
+    }
+#pragma unroll 1
+    for (int jb = first; jb < wcols; jb += U * T) {
+        double vk[U], vp[U], u[U];
+#pragma unroll
+        for (int c = 0; c < U; ++c) {
+            const int j = jb + t + c * T;
+            const bool in = j < wcols;
+            vk[c] = in ? TL_SM(M, rk + j, lim) : 0.0;
+            vp[c] = in ? TL_SM(M, rp + j, lim) : 0.0;
+            if (PEND) u[c] = in ? TL_SM(M, ru + j, lim) : 0.0;
         }
+#pragma unroll
+        for (int c = 0; c < U; ++c) {
+            // a branch the whole warp takes: an FP64 instruction of which no
+            // lane is active still takes the pipe for its 64 clocks
+            if (jb + c * T >= wcols) break;
+            const int j = jb + t + c * T;
+            const unsigned hi = static_cast<unsigned>(dev::mag_bits(vp[c]) >> 32);
+            worst = (j < n && hi > worst) ? hi : worst;
+            if (PEND) vp[c] = dev::sel(upd, __fma_rn(l, u[c], vp[c]), vp[c]);
+            if (j < wcols) {
+                TL_SM(M, rp + j, lim) = vk[c];
+                TL_SM(M, rk + j, lim) = vp[c];
+            }
+        }
+        if (U * T > TL_MAX_N) break;
     }
 }
 
+// Multiplier of a step whose pivot is zero (a sign flip) or below DBL_MIN
+// (a quotient) in some group of the warp; out of line.
+static __device__ __noinline__ double smem_rare_multiplier(double a, double cv, double nr, bool zero, bool small)
+{
+    return zero ? dev::neg(a) : small ? __ddiv_rn(a, dev::neg(cv)) : __dmul_rn(a, nr);
+}
+
+// Negated multipliers of column k below row k; with UPD the same lane also
+// applies step k to the entry of column k + 1 of its row and proposes it as a
+// pivot candidate of step k + 1 (rows below hi).
+template <int T, bool UPD>
+__device__ __forceinline__ void smem_multipliers(double *M, int n, int RS, int k, int t, int lim, double cv, double nr,
+                                                 bool zero, bool small, int hi, PivotScan &sc)
+{
+    constexpr int U = RowChunk<T>::U;
+    const double ukk1 = UPD ? TL_SM(M, k * RS + k + 1, lim) : 0.0;
+    const bool rare = __any_sync(0xffffffffu, small || zero);
+    if (UPD) sc.clear();
+#pragma unroll 1
+    for (int ib = k + 1; ib < n; ib += U * T) {
+        double a[U], b[U];
+#pragma unroll
+        for (int c = 0; c < U; ++c) {
+            const int i = ib + t + c * T;
+            a[c] = i < n ? TL_SM(M, i * RS + k, lim) : 0.0;
+            if (UPD) b[c] = i < n ? TL_SM(M, i * RS + k + 1, lim) : 0.0;
+        }
+#pragma unroll
+        for (int c = 0; c < U; ++c) {
+            if (ib + c * T >= n) break;  // the same on every lane
+            const int i = ib + t + c * T;
+            const double l = rare ? smem_rare_multiplier(a[c], cv, nr, zero, small) : __dmul_rn(a[c], nr);
+            if (i < n) TL_SM(M, i * RS + k, lim) = l;
+            if (UPD) {
+                const double w = dev::sel(zero, b[c], __fma_rn(l, ukk1, b[c]));
+                if (i < n) TL_SM(M, i * RS + k + 1, lim) = w;
+                sc.add(w, i, i < hi);
+            }
+        }
+        if (U * T >= TL_MAX_N) break;
+    }
+}
+
+// Returns info; worst receives the largest high word of the magnitudes of
+// A's entries and of the values that replaced them, as this lane met them: a
+// non-finite entry of A stays non-finite until it is in a pivot column or in
+// a row of U, so only when some lane of the group reports 0x7ff00000 or more
+// can A hold one.
 template <int T, bool SOLVE, bool KEEPL>
-__device__ __forceinline__ int smem_lupp2(double *M, int n, int RS, int t, int tile, double threshold)
+__device__ __forceinline__ int smem_lupp2(double *M, int n, int RS, int t, int tile, double threshold, unsigned &worst)
 {
     static_assert(T >= 1 && T <= 32 && (32 % T) == 0, "T must divide 32");
     const int lane0 = (static_cast<int>(threadIdx.x) & 31) - t;
@@ -445,38 +550,51 @@ __device__ __forceinline__ int smem_lupp2(double *M, int n, int RS, int t, int t
     int *piv = reinterpret_cast<int *>(rcp + n);        // n ints
     int info = 0;
     bool tiny = false;
+    worst = 0;
     const int wcols = n + (SOLVE ? 1 : 0);              // columns incl. b
+    auto note = [&](double v) {
+        const unsigned hi = static_cast<unsigned>(dev::mag_bits(v) >> 32);
+        worst = hi > worst ? hi : worst;
+    };
+    PivotScan sc;
     int k = 0;
     for (; k + 1 < n; k += 2) {
-        // ---- step k: pivot, interchange, multipliers, column k+1 ----
+        // ---- step k: pivot, reciprocal and interchange, multipliers, column
+        //      k+1 with the candidates of step k+1 ----
+        const int hi0 = smem_pivot_limit(n, k, tile);
+        smem_scan<T>(M, RS, k, k, hi0, t, lim, sc);
         double cv;
-        smem_pivot_step<T>(M, n, RS, k, t, lim, KEEPL ? 0 : k, wcols, tile, threshold, piv, cv, info);
+        int p;
+        smem_pivot<T>(M, n, RS, k, hi0, t, lim, threshold, sc, piv, cv, p, info);
+        note(cv);
         const bool z0 = dev::mag_bits(cv) == 0ULL;
         const bool s0 = !z0 && dev::mag_bits(cv) < dev::kDblMinBits;
+        smem_swap<T, false>(M, n, RS, k, p, t, lim, KEEPL ? 0 : k, wcols, 0.0, false, worst);
         const double r0 = dev::rcp_rn(cv);
         if (t == 0) TL_SM(rcp, k, n) = r0;
         tiny = tiny || s0;
         __syncwarp();
-        smem_multipliers<T, true>(M, n, RS, k, t, lim, cv, dev::neg(r0), z0, s0);
-        __syncwarp();
-        // ---- step k+1: pivot (column k+1 is up to date), interchange rows
-        //      that still carry step k's pending update and -l_ik ----
         const int k1 = k + 1;
+        const int hi1 = smem_pivot_limit(n, k1, tile);
+        smem_multipliers<T, true>(M, n, RS, k, t, lim, cv, dev::neg(r0), z0, s0, hi1, sc);
+        __syncwarp();
+        // ---- step k+1: pivot, interchange of rows that still carry step k's
+        //      pending update and -l_ik (the new row k+1 receives it on the
+        //      way), multipliers ----
         double cv1;
-        smem_pivot_step<T>(M, n, RS, k1, t, lim, KEEPL ? 0 : k, wcols, tile, threshold, piv, cv1, info);
+        int p1;
+        smem_pivot<T>(M, n, RS, k1, hi1, t, lim, threshold, sc, piv, cv1, p1, info);
+        note(cv1);
         const bool z1 = dev::mag_bits(cv1) == 0ULL;
         const bool s1 = !z1 && dev::mag_bits(cv1) < dev::kDblMinBits;
+        const double lp = TL_SM(M, p1 * RS + k, lim);
+        __syncwarp();
+        smem_swap<T, true>(M, n, RS, k1, p1, t, lim, KEEPL ? 0 : k, wcols, lp, !z0, worst);
         const double r1 = dev::rcp_rn(cv1);
         if (t == 0) TL_SM(rcp, k1, n) = r1;
         tiny = tiny || s1;
         __syncwarp();
-        // row k+1 receives step k (columns k+2..); column k+1 its multipliers
-        if (!z0) {
-            const double l = TL_SM(M, k1 * RS + k, lim);
-            for (int j = k + 2 + t; j < wcols; j += T)
-                TL_SM(M, k1 * RS + j, lim) = __fma_rn(l, TL_SM(M, k * RS + j, lim), TL_SM(M, k1 * RS + j, lim));
-        }
-        smem_multipliers<T, false>(M, n, RS, k1, t, lim, cv1, dev::neg(r1), z1, s1);
+        smem_multipliers<T, false>(M, n, RS, k1, t, lim, cv1, dev::neg(r1), z1, s1, n, sc);
         __syncwarp();
         // ---- both updates of the block rows k+2.., columns k+2.. ----
         const int ncols = wcols - (k + 2);
@@ -520,12 +638,16 @@ __device__ __forceinline__ int smem_lupp2(double *M, int n, int RS, int t, int t
         }
         __syncwarp();
     }
-    if (k < n) {  // odd n: the last step (one row: its pivot and reciprocal)
-        double cv;
-        smem_pivot_step<T>(M, n, RS, k, t, lim, KEEPL ? 0 : k, wcols, tile, threshold, piv, cv, info);
+    if (k < n) {  // odd n: the last step (one row: its own pivot)
+        const double cv = TL_SM(M, k * RS + k, lim);
+        note(cv);
+        if (dev::mag_bits(cv) == 0ULL && info == 0) info = k + 1;
         const bool s0 = dev::mag_bits(cv) != 0ULL && dev::mag_bits(cv) < dev::kDblMinBits;
         const double r0 = dev::rcp_rn(cv);
-        if (t == 0) TL_SM(rcp, k, n) = r0;
+        if (t == 0) {
+            TL_SM(piv, k, n) = k;
+            TL_SM(rcp, k, n) = r0;
+        }
         tiny = tiny || s0;
         __syncwarp();
     }
@@ -535,21 +657,34 @@ __device__ __forceinline__ int smem_lupp2(double *M, int n, int RS, int t, int t
     if (SOLVE) {
         const bool any_tiny = __any_sync(0xffffffffu, tiny);
         if constexpr (T >= 4) {
+            // y in registers (lane t holds rows t, t + T, ...); the next
+            // column of U and the next reciprocal are loaded before the
+            // product of the current row
             constexpr int KM = TL_MAX_N / T;  // row slots per lane
-            double y[KM];
+            double y[KM], u[KM];
 #pragma unroll
             for (int s = 0; s < KM; ++s) {
                 const int r = t + s * T;
                 y[s] = r < n ? TL_SM(M, r * RS + n, lim) : 0.0;
+                u[s] = r < n - 1 ? TL_SM(M, r * RS + n - 1, lim) : 0.0;
             }
+            double rc = TL_SM(rcp, n - 1, n);
+#pragma unroll 1
             for (int i = n - 1; i >= 0; --i) {
                 const int owner = i % T, slot = i / T;
                 double yi = y[0];
 #pragma unroll
                 for (int s = 1; s < KM; ++s) yi = dev::sel(s == slot, y[s], yi);
                 double xi;
-                if (!any_tiny) xi = __dmul_rn(yi, TL_SM(rcp, i, n));
-                else xi = tiny ? __ddiv_rn(yi, TL_SM(M, i * RS + i, lim)) : __dmul_rn(yi, TL_SM(rcp, i, n));
+                if (!any_tiny) xi = __dmul_rn(yi, rc);
+                else xi = tiny ? __ddiv_rn(yi, TL_SM(M, i * RS + i, lim)) : __dmul_rn(yi, rc);
+                double un[KM];
+#pragma unroll
+                for (int s = 0; s < KM; ++s) {
+                    const int r = t + s * T;
+                    un[s] = r < i - 1 ? TL_SM(M, r * RS + i - 1, lim) : 0.0;
+                }
+                rc = TL_SM(rcp, i > 0 ? i - 1 : 0, n);
                 xi = __shfl_sync(0xffffffffu, xi, lane0 + owner);
 #pragma unroll
                 for (int s = 0; s < KM; ++s) y[s] = dev::sel(t == owner && s == slot, xi, y[s]);
@@ -557,9 +692,10 @@ __device__ __forceinline__ int smem_lupp2(double *M, int n, int RS, int t, int t
 #pragma unroll
                 for (int s = 0; s < KM; ++s) {
                     if (s * T >= i) break;  // no row of this slot lies above row i
-                    const int r = t + s * T;
-                    if (r < i) y[s] = __fma_rn(TL_SM(M, r * RS + i, lim), nxi, y[s]);
+                    if (t + s * T < i) y[s] = __fma_rn(u[s], nxi, y[s]);
                 }
+#pragma unroll
+                for (int s = 0; s < KM; ++s) u[s] = un[s];
             }
 #pragma unroll
             for (int s = 0; s < KM; ++s) {
@@ -587,9 +723,22 @@ __device__ __forceinline__ int smem_lupp2(double *M, int n, int RS, int t, int t
     return info;
 }
 
+// Whether some entry of a group's system (nn consecutive doubles at A, null
+// without a system) is not finite, read only when some group of the warp
+// suspects it (see smem_lupp2).
+template <int T>
+__device__ __forceinline__ bool smem_bad_input(bool suspect, const double *A, int nn, int t)
+{
+    if (!__any_sync(0xffffffffu, suspect)) return false;
+    int badv = 0;
+    if (A)
+        for (int e = t; e < nn; e += T) badv |= dev::is_nonfinite(A[e]) ? 1 : 0;
+    return group_any_int<T>(badv) != 0;
+}
+
 // MODE: kGesv (A const, b -> x, LU optional by KEEP) or kGetrf (A in place).
 // WALK: element walk of the trailing update instead of the lane tile.
-template <int T, int LAYOUT, int MODE, bool KEEP, bool WALK = (T >= 16), bool ASYNC_LOAD = (T < 16)>
+template <int T, int LAYOUT, int MODE, bool KEEP, bool WALK = (T >= 16)>
 __global__ void __launch_bounds__(128) k_smem_group(SolveArgs args, int n)
 {
     extern __shared__ double smem[];
@@ -601,47 +750,37 @@ __global__ void __launch_bounds__(128) k_smem_group(SolveArgs args, int n)
     const int nn = n * n;
     const unsigned m20 = magic20(n);
 
-    // ---- load: thread (q = tid % SB, t' = tid / SB) copies elements
-    //      e = t', t'+T, ... of system s0+q (coalesced over q): cp.async,
-    //      or register-staged streaming loads (ASYNC_LOAD false) ----
-    {
+    // ---- load, all copies in flight at once (cp.async).  Interleaved: thread
+    //      (q = tid % SB, tp = tid / SB) copies entries tp, tp+T, ... of
+    //      system s0+q (coalesced over q); per system: a warp copies 32
+    //      consecutive entries of one system at a time ----
+    if (LAYOUT == kInterleaved) {
         const int q = threadIdx.x % SB;
         const int tp = threadIdx.x / SB;
         const int64_t s = s0 + q;
         double *M = smem + q * per;
-        if (!ASYNC_LOAD && s < args.batch) {
-            const double *src = Ag + (LAYOUT == kInterleaved ? s : s * nn);
-            const int64_t es = LAYOUT == kInterleaved ? args.ld : 1;
-#pragma unroll 4
+        if (s < args.batch) {
             for (int e = tp; e < nn; e += T) {
                 const int j = div20(e, m20);
-                TL_SM(M, (e - j * n) * RS + j, per) = ld_stream(src + e * es);
+                cp_async8(&TL_SM(M, (e - j * n) * RS + j, per), Ag + static_cast<int64_t>(e) * args.ld + s);
             }
-            if (MODE == kGesv) {
-                const double *bs = args.b + (LAYOUT == kInterleaved ? s : s * n);
-                for (int i2 = tp; i2 < n; i2 += T) TL_SM(M, i2 * RS + n, per) = ld_stream(bs + i2 * es);
-            }
-        } else if (s < args.batch) {
-            if (LAYOUT == kInterleaved) {
-                for (int e = tp; e < nn; e += T) {
-                    const int j = div20(e, m20);
-                    cp_async8(&TL_SM(M, (e - j * n) * RS + j, per), Ag + static_cast<int64_t>(e) * args.ld + s);
-                }
-                if (MODE == kGesv)
-                    for (int i2 = tp; i2 < n; i2 += T)
-                        cp_async8(&TL_SM(M, i2 * RS + n, per), args.b + static_cast<int64_t>(i2) * args.ld + s);
-            } else {
-                const double *src = Ag + s * nn;
-                for (int e = tp; e < nn; e += T) {
-                    const int j = div20(e, m20);
-                    cp_async8(&TL_SM(M, (e - j * n) * RS + j, per), src + e);
-                }
-                if (MODE == kGesv)
-                    for (int i2 = tp; i2 < n; i2 += T) cp_async8(&TL_SM(M, i2 * RS + n, per), args.b + s * n + i2);
-            }
+            if (MODE == kGesv)
+                for (int i2 = tp; i2 < n; i2 += T)
+                    cp_async8(&TL_SM(M, i2 * RS + n, per), args.b + static_cast<int64_t>(i2) * args.ld + s);
         }
-        cp_async_wait_all();
+    } else {
+        const int lane = threadIdx.x & 31;
+        for (int q = threadIdx.x >> 5; q < SB && s0 + q < args.batch; q += blockDim.x >> 5) {
+            double *M = smem + q * per;
+            const double *src = Ag + (s0 + q) * nn;
+            for (int e = lane; e < nn; e += 32) {
+                const int j = div20(e, m20);
+                cp_async8(&TL_SM(M, (e - j * n) * RS + j, per), src + e);
+            }
+            if (MODE == kGesv && lane < n) cp_async8(&TL_SM(M, lane * RS + n, per), args.b + (s0 + q) * n + lane);
+        }
     }
+    cp_async_wait_all();
     __syncthreads();
 
     // ---- compute: lanes t = lane % T of a group own system q ----
@@ -652,22 +791,34 @@ __global__ void __launch_bounds__(128) k_smem_group(SolveArgs args, int n)
     const bool active = s < args.batch;
     double *M = smem + q * per;
     const int *piv = reinterpret_cast<const int *>(M + smem_piv_offset(n));  // pivots (after n reciprocals)
-    // non-finite entries anywhere in this system
-    int badv = 0;
-    if (active) {
-        for (int e = t; e < nn; e += T) {
-            const int j = div20(e, m20);
-            badv |= dev::is_nonfinite(M[(e - j * n) * RS + j]) ? 1 : 0;
+    bool bad = false;
+    int info;
+    if constexpr (WALK) {
+        unsigned worst = 0;
+        info = smem_lupp2<T, MODE == kGesv, KEEP || MODE == kGetrf>(M, n, RS, t, args.tile, args.threshold, worst);
+        // only a system that met a non-finite value can have one in A; whether
+        // it has (or overflowed on the way) is read from A again
+        const bool suspect = active && worst >= 0x7ff00000u;
+        if (__any_sync(0xffffffffu, suspect)) {
+            int badv = 0;
+            if (active) {
+                const double *src = Ag + (LAYOUT == kInterleaved ? s : s * nn);
+                const int64_t es = LAYOUT == kInterleaved ? args.ld : 1;
+                for (int e = t; e < nn; e += T) badv |= dev::is_nonfinite(src[e * es]) ? 1 : 0;
+            }
+            bad = group_any_int<T>(badv) != 0;
         }
+    } else {
+        int badv = 0;
+        if (active) {
+            for (int e = t; e < nn; e += T) {
+                const int j = div20(e, m20);
+                badv |= dev::is_nonfinite(M[(e - j * n) * RS + j]) ? 1 : 0;
+            }
+        }
+        bad = group_any_int<T>(badv) != 0;
+        info = smem_lupp<T, MODE == kGesv, false>(M, n, RS, t, args.tile, args.threshold);
     }
-    const bool bad = group_any_int<T>(badv) != 0;
-
-    int info0;
-    if constexpr (WALK)
-        info0 = smem_lupp2<T, MODE == kGesv, KEEP || MODE == kGetrf>(M, n, RS, t, args.tile, args.threshold);
-    else
-        info0 = smem_lupp<T, MODE == kGesv, false>(M, n, RS, t, args.tile, args.threshold);
-    int info = info0;
     if (bad) info = -1;
 
     // a7: store
@@ -740,15 +891,10 @@ __global__ void __launch_bounds__(128) k_smem_ragged(RaggedArgs r, int n)
         __syncthreads();
         const bool active = base + q < count;
         double *M = smem + q * per;
-        int badv = 0;
-        if (active) {
-            for (int e = t; e < nn; e += T) {
-                const int j = div20(e, m20);
-                badv |= dev::is_nonfinite(M[(e - j * n) * RS + j]) ? 1 : 0;
-            }
-        }
-        const bool bad = group_any_int<T>(badv) != 0;
-        int info = smem_lupp2<T, true, false>(M, n, RS, t, 0, 0.0);
+        unsigned worst = 0;
+        int info = smem_lupp2<T, true, false>(M, n, RS, t, 0, 0.0, worst);
+        const bool bad = smem_bad_input<T>(active && worst >= 0x7ff00000u,
+                                           active ? r.A + r.a_off[r.bucket[beg + base + q]] : nullptr, nn, t);
         if (bad) info = -1;
         if (active) {
             const int64_t sidx = r.bucket[beg + base + q];
