@@ -405,7 +405,7 @@ def newton_bench(tl, h, steps, warmup, torch, device, I, seed, peak, npoints=NEW
         out["cpu_driven"] = {"ms": med_cd, "points_per_s": npoints / (med_cd / 1e3),
                              "fused_speedup": med_cd / med, "iterations": int(iters.max().item()) + 1,
                              "results_equal_fused": same,
-                             "launches_per_iteration": "assemble + gesv (+ fixup) + update, D2H count"}
+                             "launches_per_iteration": "assemble + gesv + update, D2H count"}
         del x_f, it_f, st_f
     return out
 
@@ -588,7 +588,7 @@ def ragged_bench(tl, h, steps, warmup, torch, device, I, seed, batch=RAGGED_BATC
     med = timed(run_plain)
     same = all(torch.equal(q["p"], piv_ref[d["buckets"][n][2]]) for n, q in per_n.items())
     out["fp64_plain_per_n_gesv"] = {"ms": med, "solves_per_s": batch / (med / 1e3),
-                                    "launches": f"{len(per_n)} tl_gesv_batched (+ fixup passes)",
+                                    "launches": f"{len(per_n)} tl_gesv_batched",
                                     "pivots_equal_persistent": same,
                                     "inputs": "pre-bucketed contiguous per-n copies (bucketing not timed)"}
 
@@ -1048,9 +1048,8 @@ def main():
                          "per-n batch sizes"}
 
     log("done")
-    # one launch per n and step, plus the fixup launch that follows the
-    # one-thread register kernels (variant 1) on the same stream
-    launches = sum(2 if tl.tl_dispatch_get(h, n, 1)[1] == 1 else 1 for n in n_list) * args.steps
+    # one launch per n and step
+    launches = len(n_list) * args.steps
     tl.tl_destroy(h)
     if rank == 0:
         out = {

@@ -56,7 +56,8 @@ SPILL_ALLOW = [
     # registers as well; tuned dispatch runs the shared-memory solver there
     (r"k_factor_groupILi\d+ELi\d+ELi\d+ELi\d+ELb1E", 640, 640),
     (r"k_factor_groupILi23ELi8E", 16, 16),
-    (r"k_fixup_thread|k_getrs_thread", 32, 32),
+    # the calls of the exact general path, out of line
+    (r"slow_factor_thread|slow_ragged_thread|k_getrs_thread|k_factor_threadILi[678]E|k_ragged_threadILi[89]E", 64, 64),
     (r"k_ragged_irILi1[34]ELi4E", 64, 64),
     # shared-memory solvers: ptxas parks a few addresses of the load and
     # store phases on the stack (the same with a higher register limit);

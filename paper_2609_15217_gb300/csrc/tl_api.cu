@@ -39,13 +39,13 @@ static VariantList g_registry[TL_MAX_N + 1][2][kOps];
 
 VariantList &registry(int n, int layout, int op) { return g_registry[n][layout][op]; }
 
-void register_variant(int n, int layout, int op, int lanes, const void *kernel, int kind, const void *fixup)
+void register_variant(int n, int layout, int op, int lanes, const void *kernel, int kind, int warp_smem)
 {
     if (n < 1 || n > TL_MAX_N || layout < 0 || layout > 1 || op < 0 || op >= kOps) return;
     VariantList &l = g_registry[n][layout][op];
     for (int i = 0; i < l.count; ++i)
         if (l.v[i].lanes == lanes && l.v[i].kind == kind) return;
-    if (l.count < kMaxVariants) l.v[l.count++] = Variant{lanes, kernel, kind, fixup};
+    if (l.count < kMaxVariants) l.v[l.count++] = Variant{lanes, kernel, kind, warp_smem};
 }
 
 // Default thread-to-system mapping per n before any autotuning: one thread
@@ -212,29 +212,26 @@ tl_status launch_variant(tl_handle *h, const Variant *v, int n, int block, Solve
 {
     if (args.batch == 0) return TL_OK;
     const int64_t threads = args.batch * v->lanes;
-    const size_t per_sys = v->kind >= 1 ? smem_sys_bytes(n, v->lanes) : 0;
+    const bool shared = v->kind == 1 || v->kind == 2;
+    const size_t per_sys = shared ? smem_sys_bytes(n, v->lanes) : static_cast<size_t>(v->warp_smem) * v->lanes / 32;
     cudaError_t e;
     int dyn_limit = h->max_smem_per_block;
-    if (v->kind >= 1) {
+    if (per_sys) {
         const tl_status st = smem_opt_in(h, v->kernel, &dyn_limit);
         if (st != TL_OK) return st;
     }
     if (block <= 0) block = pick_block(h, v->kernel, threads, v->lanes, per_sys, dyn_limit);
     const int64_t grid = (threads + block - 1) / block;
     if (grid > INT_MAX) return TL_ERR_UNSUPPORTED;
-    if (v->kind >= 1) {
-        const size_t smem = (block / v->lanes) * per_sys;
-        if (smem > static_cast<size_t>(dyn_limit)) return TL_ERR_UNSUPPORTED;
+    const size_t smem = (block / v->lanes) * per_sys;
+    if (smem > static_cast<size_t>(dyn_limit)) return TL_ERR_UNSUPPORTED;
+    if (shared) {
         int nn = n;
         void *params[] = {&args, &nn};
         e = cudaLaunchKernel(v->kernel, dim3(static_cast<unsigned>(grid)), dim3(block), params, smem, stream);
     } else {
         void *params[] = {&args};
-        e = cudaLaunchKernel(v->kernel, dim3(static_cast<unsigned>(grid)), dim3(block), params, 0, stream);
-        if (e == cudaSuccess && v->fixup) {
-            const int64_t fgrid = (args.batch + 127) / 128;
-            e = cudaLaunchKernel(v->fixup, dim3(static_cast<unsigned>(fgrid)), dim3(128), params, 0, stream);
-        }
+        e = cudaLaunchKernel(v->kernel, dim3(static_cast<unsigned>(grid)), dim3(block), params, smem, stream);
     }
     if (e != cudaSuccess) return fail_cuda(h, e);
     return TL_OK;

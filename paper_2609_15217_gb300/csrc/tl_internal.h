@@ -62,7 +62,7 @@ struct Variant {
     int lanes;                     // T
     const void *kernel;            // __global__ function, for occupancy queries
     int kind;
-    const void *fixup;             // second pass for flagged systems (or null)
+    int warp_smem;                 // kind 0: dynamic shared memory per warp in bytes
 };
 __host__ __device__ constexpr int variant_id(int lanes, int kind) { return lanes + 100 * kind; }
 
@@ -84,6 +84,6 @@ struct VariantList {
 };
 VariantList &registry(int n, int layout, int op);
 void register_variant(int n, int layout, int op, int lanes, const void *kernel, int kind = 0,
-                      const void *fixup = nullptr);
+                      int warp_smem = 0);
 
 }  // namespace tl

@@ -27,11 +27,6 @@ struct Idx {
     }
 };
 
-// info value the fast one-thread kernels leave for a system that must be
-// redone by the exact general path; the fixup kernel that runs right after
-// them on the same stream replaces it, so callers never see it.
-constexpr int32_t kInfoSlow = -2147483000;
-
 // Streaming loads/stores: every input is read once and every output written
 // once, so keep them out of the way of the L2 lines that are reused.
 __device__ __forceinline__ double ld_stream(const double *p) { return __ldcs(p); }
@@ -65,9 +60,12 @@ __device__ __forceinline__ int div20(int x, unsigned m) { return static_cast<int
 // ---------------------------------------------------------------------------
 // Exact general path for one system (zero, tiny, huge or non-finite pivots
 // or inputs): loads the system again, factors it with lu_thread_factor and
-// stores every output.
+// stores every output.  Out of line, so that its registers do not weigh on the
+// fast path; a second launch over the systems the first one flagged, which
+// this replaced, cost 15 of 351 us at n = 7, 1,000,003 systems, and 3 of
+// 10 us at 64.
 template <int N, int LAYOUT, int MODE, bool KEEP>
-__device__ __forceinline__ void slow_factor_thread(SolveArgs args, int64_t s)
+__device__ __noinline__ void slow_factor_thread(SolveArgs args, int64_t s)
 {
     using I = Idx<N, LAYOUT>;
     const double *A = (MODE == kGetrf) ? args.LU : args.A;
@@ -110,30 +108,76 @@ __device__ __forceinline__ void slow_factor_thread(SolveArgs args, int64_t s)
     args.info[s] = info;
 }
 
+// Per-system storage from n = 8 on: a thread's own entries are n^2 doubles
+// from its neighbour's, so a warp reads its 32 consecutive systems as one
+// run of memory (cp.async) into shared memory and takes them from there
+// (odd stride: no bank conflict).  1,048,576 systems of n = 8: 0.69 TFLOP/s
+// with direct loads, against 0.86 interleaved; below n = 8 the caches do it.
+template <int N, int LAYOUT>
+constexpr bool kThreadStaged = LAYOUT == kPerSystem && N >= 8;
+__host__ __device__ constexpr int thread_stage_stride(int n) { return (n * n + n) | 1; }
+__host__ __device__ constexpr int thread_stage_doubles(int n) { return 32 * thread_stage_stride(n); }
+
+// Resident blocks asked of the compiler: 168 registers at n = 7, without
+// which the integer reciprocal takes 190 and a third of the warps (0.87 ->
+// 0.62 TFLOP/s).
+constexpr int thread_min_blocks(int n) { return n == 7 ? 3 : 0; }
+
 template <int N, int LAYOUT, int MODE, bool KEEP>
-__global__ void __launch_bounds__(128) k_factor_thread(SolveArgs args)
+__global__ void __launch_bounds__(128, KEEP ? 0 : thread_min_blocks(N)) k_factor_thread(SolveArgs args)
 {
     const int64_t s = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (s >= args.batch) return;
     using I = Idx<N, LAYOUT>;
     const double *A = (MODE == kGetrf) ? args.LU : args.A;
     double a[N][N];
-#pragma unroll
-    for (int j = 0; j < N; ++j)
-#pragma unroll
-        for (int i = 0; i < N; ++i) a[i][j] = (MODE == kGetrf) ? A[I::a(s, i, j, args.ld)]
-                                                                 : ld_stream(A + I::a(s, i, j, args.ld));
     double b[1][N];
-    if (MODE == kGesv) {
+    if constexpr (kThreadStaged<N, LAYOUT>) {
+        extern __shared__ double stage[];
+        constexpr int NN = N * N, ST = thread_stage_stride(N);
+        const int lane = threadIdx.x & 31;
+        double *W = stage + (threadIdx.x >> 5) * thread_stage_doubles(N);
+        const int64_t s0 = s - lane;
+        if (s0 >= args.batch) return;  // the whole warp
+        const int live = static_cast<int>(args.batch - s0 < 32 ? args.batch - s0 : 32);
+        const double *src = A + s0 * NN;
+        for (int e = lane; e < live * NN; e += 32) cp_async8(W + (e / NN) * ST + e % NN, src + e);
+        if (MODE == kGesv) {
+            const double *bs = args.b + s0 * N;
+            for (int e = lane; e < live * N; e += 32) cp_async8(W + (e / N) * ST + NN + e % N, bs + e);
+        }
+        cp_async_wait_all();
+        __syncwarp();
+        if (s >= args.batch) return;
+        const double *M = W + lane * ST;
 #pragma unroll
-        for (int i = 0; i < N; ++i) b[0][i] = ld_stream(args.b + I::v(s, i, args.ld));
+        for (int j = 0; j < N; ++j)
+#pragma unroll
+            for (int i = 0; i < N; ++i) a[i][j] = M[j * N + i];
+        if (MODE == kGesv) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) b[0][i] = M[NN + i];
+        }
+    } else {
+        if (s >= args.batch) return;
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+#pragma unroll
+            for (int i = 0; i < N; ++i) a[i][j] = (MODE == kGetrf) ? A[I::a(s, i, j, args.ld)]
+                                                                     : ld_stream(A + I::a(s, i, j, args.ld));
+        if (MODE == kGesv) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) b[0][i] = ld_stream(args.b + I::v(s, i, args.ld));
+        }
     }
     // Branch-free fast path; a system with a zero, tiny, huge or non-finite
     // pivot (or input) is redone from its input by the exact general path.
     const bool bad = dev::any_nonfinite<N>(a);
     int piv[N];
     double rcp[N];
-    const bool slow = dev::lu_thread_factor_fast<N, KEEP, (MODE == kGesv) ? 1 : 0>(a, b, piv, rcp) || bad;
+    // (with L kept, 6 and more rows have no registers left for the integer
+    // reciprocal)
+    constexpr bool RCP_INT = N <= (KEEP ? 5 : TL_THREAD_RCP_INT_MAX_N);
+    const bool slow = dev::lu_thread_factor_fast<N, KEEP, (MODE == kGesv) ? 1 : 0, RCP_INT>(a, b, piv, rcp) || bad;
     if (!slow) {
         if (MODE == kGesv) {
             dev::lu_thread_backsolve_fast<N>(a, b[0], rcp);
@@ -151,20 +195,8 @@ __global__ void __launch_bounds__(128) k_factor_thread(SolveArgs args)
         for (int k = 0; k < N; ++k) st_stream(args.ipiv + I::v(s, k, args.ld), piv[k] + 1);
         st_stream(args.info + s, 0);
     } else {
-        args.info[s] = kInfoSlow;  // redone by k_fixup_thread
+        slow_factor_thread<N, LAYOUT, MODE, KEEP>(args, s);
     }
-}
-
-// Second pass after k_factor_thread: the systems it flagged go through the
-// exact general path.  A separate kernel so that the general path's registers
-// never weigh on the fast kernel.
-template <int N, int LAYOUT, int MODE, bool KEEP>
-__global__ void __launch_bounds__(128) k_fixup_thread(SolveArgs args)
-{
-    const int64_t s = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (s >= args.batch) return;
-    if (args.info[s] != kInfoSlow) return;
-    slow_factor_thread<N, LAYOUT, MODE, KEEP>(args, s);
 }
 
 // One thread per system: solve with given factors, nrhs right-hand sides.
@@ -376,7 +408,7 @@ __device__ __forceinline__ int64_t ragged_count(const RaggedArgs &r, int64_t beg
 
 // Exact general path of one ragged system (see slow_factor_thread).
 template <int N>
-__device__ __forceinline__ void slow_ragged_thread(RaggedArgs r, int64_t s)
+__device__ __noinline__ void slow_ragged_thread(RaggedArgs r, int64_t s)
 {
     const double *A = r.A + r.a_off[s];
     const double *bv = r.b + r.b_off[s];
@@ -436,20 +468,8 @@ __global__ void __launch_bounds__(128) k_ragged_thread(RaggedArgs r)
             for (int k = 0; k < N; ++k) st_stream(ip + k, piv[k] + 1);
             st_stream(r.info + s, 0);
         } else {
-            r.info[s] = kInfoSlow;  // redone by k_ragged_fixup
+            slow_ragged_thread<N>(r, s);
         }
-    }
-}
-
-template <int N>
-__global__ void __launch_bounds__(128) k_ragged_fixup(RaggedArgs r)
-{
-    const int64_t beg = r.offsets[N];
-    const int64_t count = ragged_count<N>(r, beg);
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < count; q += stride) {
-        const int64_t s = r.bucket[beg + q];
-        if (r.info[s] == kInfoSlow) slow_ragged_thread<N>(r, s);
     }
 }
 

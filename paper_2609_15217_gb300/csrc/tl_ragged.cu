@@ -269,8 +269,7 @@ tl_status launch_per_size(tl_handle *h, RaggedArgs &r, cudaStream_t stream, int6
         const int blk = 128;
         const unsigned g = ragged_grid(h, v, batch, blk);
         void *params[] = {&r};
-        cudaError_t e = cudaLaunchKernel(v->kernel, dim3(g), dim3(blk), params, 0, stream);
-        if (e == cudaSuccess && v->fixup) e = cudaLaunchKernel(v->fixup, dim3(g), dim3(blk), params, 0, stream);
+        const cudaError_t e = cudaLaunchKernel(v->kernel, dim3(g), dim3(blk), params, 0, stream);
         if (e != cudaSuccess) return fail_cuda(h, e);
     }
     return TL_OK;

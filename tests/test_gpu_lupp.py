@@ -185,3 +185,30 @@ def test_argument_errors(tl, h):
     assert tl.tl_last_bad_arg(h) == 3
     assert tl.tl_getrf_batched(h, 4, d.data_ptr() + 4, 0, 0, i, i, 1) == tl.TL_ERR_INVALID_ARG
     assert tl.tl_last_bad_arg(h) == 3           # misaligned
+
+
+@pytest.mark.parametrize("layout", [0, 1], ids=["per_system", "interleaved"])
+@pytest.mark.parametrize("n", list(range(1, 10)))
+def test_one_thread_kernels(tl, h, n, layout):
+    """The one-thread register kernels at a batch that ends inside a warp and
+    inside a block, with systems that take the exact general path (zero,
+    subnormal, huge and non-finite entries) next to ordinary ones."""
+    batch = 2 * 128 + 45
+    A, b, _, _ = inputs.sweep_systems(n, batch, 6200 + n)
+    A[3, :, n // 2] = 0.0
+    A[35, n - 1, 0] = np.nan
+    A[36] *= 2.0 ** -1060
+    A[130, 0, 0] = 1e308
+    A[batch - 1, 0, n - 1] = np.inf
+    x_o, piv_o, info_o, _, LU_o = oracle.gesv(A, b, want_lu=True)
+    assert tl.tl_dispatch_set(h, n, layout, 1, 0) == tl.TL_OK
+    try:
+        x_g, piv_g, info_g, LU_g = gpu_gesv(tl, h, A, b, layout)
+        x_2, piv_2, info_2, _ = gpu_gesv(tl, h, A, b, layout, want_lu=False)
+    finally:
+        tl.tl_dispatch_set(h, n, layout, 0, 0)
+    ok = info_o >= 0
+    assert np.array_equal(info_g, info_o) and np.array_equal(info_2, info_o)
+    assert np.array_equal(piv_g, piv_o) and np.array_equal(piv_2, piv_o)
+    assert np.array_equal(LU_g[ok].view(np.int64), LU_o[ok].view(np.int64))
+    assert np.array_equal(x_2, x_g, equal_nan=True) and np.isnan(x_g[info_o != 0]).all()
