@@ -77,6 +77,9 @@ KERNEL_FAMILIES = (
     + [(n, 16) for n in range(25, 33)]
 )
 
+# One row per lane (lanes >= n): the kernels of small batches.
+LATENCY_FAMILIES = [(n, 8) for n in range(5, 9)] + [(n, 16) for n in range(9, 17)]
+
 # (n, lanes per system) families of the mixed-precision (binary32 factor,
 # binary64 refinement) ragged kernel; binary32 rows take half the registers,
 # so one thread per system reaches further.
@@ -126,7 +129,7 @@ def _jobs(checked=False):
     else:
         for src in PLAIN_SOURCES:
             jobs.append((src, []))
-        for n, t in KERNEL_FAMILIES:
+        for n, t in KERNEL_FAMILIES + LATENCY_FAMILIES:
             jobs.append(("tl_inst.cu", [f"-DTL_INST_N={n}", f"-DTL_INST_T={t}"]))
         for n, t in IR_FAMILIES:
             jobs.append(("tl_inst_ir.cu", [f"-DTL_INST_N={n}", f"-DTL_INST_T={t}"]))

@@ -237,9 +237,49 @@ tl_status launch_variant(tl_handle *h, const Variant *v, int n, int block, Solve
     return TL_OK;
 }
 
+// Variant and block of a small batch (null: the large-batch default).  A
+// warp alone on a sub-partition runs at the pace of its own FP64
+// instructions and of each step's latency, so while a wider group still
+// leaves every sub-partition few warps, it is faster: fewer FP64 instructions
+// and shorter passes per warp.  n = 5..16 with one row per lane in registers
+// (8 lanes up to n = 8, else 16) up to 12 or 8 warps per SM; the element walk
+// with 32, 16, 8 or 4 lanes up to 16 warps per SM (32 lanes up to 8,192
+// systems from n = 28 on, where a wider group costs least).  Measured per call
+// in a CUDA graph, one thread per system or the large-batch lanes against
+// these: 64 systems of n = 6 7.2 -> 4.5 us; 4,096 of n = 8 14.2 -> 6.8; 1,024
+// of n = 16 35.4 -> 14.9; 256 of n = 20 36 -> 16.5; 4,096 of n = 32 154 ->
+// 127.
+static const Variant *small_batch_variant(tl_handle *h, int n, int layout, int op, int64_t batch)
+{
+    const int64_t sms = h->sm_count;
+    const int id0 = default_lanes(n, layout, op);
+    if (n <= 16) {
+        const VariantList &l = registry(n, layout, op);
+        for (int i = 0; i < l.count; ++i) {
+            const Variant *v = &l.v[i];
+            if (v->kind != kKindLatency) continue;
+            // from n = 10 on 32 lanes of the walk are faster still while
+            // there is one warp per sub-partition
+            if (n >= 10 && op != kOpGetrs && batch <= 4 * sms) break;
+            if (batch * v->lanes <= 32 * sms * (n <= 8 ? 12 : 8)) return v;
+        }
+    }
+    if (n < 10 || op == kOpGetrs) return nullptr;
+    for (int T : {32, 16, 8, 4}) {
+        if (T <= id0 % 100) break;
+        if (batch * T <= 32 * 16 * sms || (T == 32 && n >= 28 && batch <= 8192))
+            return find_variant(n, layout, op, variant_id(T, T >= 16 ? 1 : 2));
+    }
+    return nullptr;
+}
+
 tl_status launch_op(tl_handle *h, int n, int layout, int op, SolveArgs &args, cudaStream_t stream)
 {
     const Choice &c = h->choice[n][layout][op];
+    if (!c.lanes) {
+        const Variant *small = small_batch_variant(h, n, layout, op, args.batch);
+        if (small) return launch_variant(h, small, n, 32, args, stream);
+    }
     const Variant *v = find_variant(n, layout, op, c.lanes ? c.lanes : default_lanes(n, layout, op));
     if (!v) return TL_ERR_UNSUPPORTED;
     return launch_variant(h, v, n, c.lanes ? c.block : default_block(h, v, layout, args.batch), args, stream);

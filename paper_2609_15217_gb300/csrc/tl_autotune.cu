@@ -105,7 +105,7 @@ extern "C" tl_status tl_dispatch_set(tl_handle *h, int n, tl_layout layout, int 
     bool found = false;
     const VariantList &l = registry(n, layout, kOpGesv);
     for (int i = 0; i < l.count; ++i)
-        if (variant_id(l.v[i].lanes, l.v[i].kind) == variant) found = true;
+        if (l.v[i].kind != kKindLatency && variant_id(l.v[i].lanes, l.v[i].kind) == variant) found = true;
     if (!found) return fail_arg(h, 4);
     set_gesv_family(h, n, layout, variant, block);
     // the ragged kernels (binary64 and mixed precision): the register kernel
@@ -208,6 +208,7 @@ extern "C" tl_status tl_autotune(tl_handle *h, int n_min, int n_max, tl_layout l
         int best_var = 0, best_block = 0;
         for (int i = 0; i < l.count && st == TL_OK; ++i) {
             const Variant *v = &l.v[i];
+            if (v->kind == kKindLatency) continue;
             for (int block : {32, 64, 128}) {
                 if (block < v->lanes) continue;
                 if (v->kind >= 1 && (block / v->lanes) * smem_sys_bytes(n, v->lanes) + 1024 > static_cast<size_t>(h->max_smem_per_block))

@@ -23,6 +23,15 @@ void reg_one_layout()
         register_variant(N, L, kOpGesvLU, 1, reinterpret_cast<const void *>(&k_factor_thread<N, L, kGesv, true>), 0, stage);
         register_variant(N, L, kOpGetrf, 1, reinterpret_cast<const void *>(&k_factor_thread<N, L, kGetrf, true>), 0, stage);
         register_variant(N, L, kOpGetrs, 1, reinterpret_cast<const void *>(&k_getrs_thread<N, L>));
+    } else if constexpr (N <= T) {
+        // one row per lane: the kernels of small batches
+        register_variant(N, L, kOpGesv, T, reinterpret_cast<const void *>(&k_factor_group<N, T, L, kGesv, false>),
+                         kKindLatency);
+        register_variant(N, L, kOpGesvLU, T, reinterpret_cast<const void *>(&k_factor_group<N, T, L, kGesv, true>),
+                         kKindLatency);
+        register_variant(N, L, kOpGetrf, T, reinterpret_cast<const void *>(&k_factor_group<N, T, L, kGetrf, true>),
+                         kKindLatency);
+        register_variant(N, L, kOpGetrs, T, reinterpret_cast<const void *>(&k_getrs_group<N, T, L>), kKindLatency);
     } else {
         register_variant(N, L, kOpGesv, T, reinterpret_cast<const void *>(&k_factor_group<N, T, L, kGesv, false>));
         register_variant(N, L, kOpGesvLU, T, reinterpret_cast<const void *>(&k_factor_group<N, T, L, kGesv, true>));
@@ -42,7 +51,7 @@ struct Registrar {
         if constexpr (TL_INST_T == 1)
             register_variant(TL_INST_N, kPerSystem, kOpRagged, 1,
                              reinterpret_cast<const void *>(&k_ragged_thread<TL_INST_N>));
-        else if constexpr (TL_INST_N <= 16)
+        else if constexpr (TL_INST_N <= 16 && TL_INST_N > TL_INST_T)
             register_variant(TL_INST_N, kPerSystem, kOpRagged, TL_INST_T,
                              reinterpret_cast<const void *>(&k_ragged_group<TL_INST_N, TL_INST_T>));
     }

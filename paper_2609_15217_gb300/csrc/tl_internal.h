@@ -57,6 +57,9 @@ struct RaggedArgs {
 //   kind 0: register kernel compiled for one n, kernel(SolveArgs)
 //   kind 1: shared-memory kernel for any n, kernel(SolveArgs, int n) with
 //           smem_sys_bytes(n) of dynamic shared memory per system
+//   kKindLatency: register kernel compiled for one n, one row per lane
+//           (lanes >= n), kernel(SolveArgs): launched for small batches only,
+//           not a choice of the dispatch table
 // The variant id is lanes + 100 * kind.
 struct Variant {
     int lanes;                     // T
@@ -64,6 +67,7 @@ struct Variant {
     int kind;
     int warp_smem;                 // kind 0: dynamic shared memory per warp in bytes
 };
+constexpr int kKindLatency = 9;
 __host__ __device__ constexpr int variant_id(int lanes, int kind) { return lanes + 100 * kind; }
 
 // Registry filled by the instantiation units (tl_inst.cu, one per (N, T)).
@@ -77,7 +81,7 @@ enum : int {
     kOpNewtonTanh = 6
 };
 constexpr int kOps = 7;
-constexpr int kMaxVariants = 12;
+constexpr int kMaxVariants = 16;
 struct VariantList {
     int count;
     Variant v[kMaxVariants];

@@ -212,3 +212,33 @@ def test_one_thread_kernels(tl, h, n, layout):
     assert np.array_equal(piv_g, piv_o) and np.array_equal(piv_2, piv_o)
     assert np.array_equal(LU_g[ok].view(np.int64), LU_o[ok].view(np.int64))
     assert np.array_equal(x_2, x_g, equal_nan=True) and np.isnan(x_g[info_o != 0]).all()
+
+
+@pytest.mark.parametrize("n,batch", [(5, 1), (6, 7296), (8, 7296), (8, 7297), (9, 2432), (10, 608), (13, 609),
+                                     (16, 2432), (16, 2433), (20, 2432), (20, 2433), (26, 4865), (32, 8192),
+                                     (32, 8193)])
+def test_small_batch_rule(tl, h, n, batch):
+    """Both sides of the lines where the default kernel changes with the
+    batch (152 SMs): every output equal bit for bit to one fixed variant's."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(17 * n + batch)
+    for layout in (0, 1):
+        ld = L.pad_ld(batch)
+        rows = ld if layout else batch
+        A = torch.empty(n * n * rows, dtype=torch.float64, device=DEV).uniform_(-1, 1, generator=g)
+        b = torch.empty(n * rows, dtype=torch.float64, device=DEV).uniform_(-1, 1, generator=g)
+        out = []
+        for variant in (0, tl.variant_id(8, shared=True)):
+            assert tl.tl_dispatch_set(h, n, layout, variant, 0) == tl.TL_OK
+            LU, x = torch.zeros_like(A), torch.zeros_like(b)
+            piv = torch.zeros(n * rows, dtype=torch.int32, device=DEV)
+            info = torch.zeros(batch, dtype=torch.int32, device=DEV)
+            tl.check("gesv", tl.tl_gesv_batched(h, n, A, None, b, x, piv, info, layout, ld, batch), h)
+            x2 = torch.zeros_like(b)
+            tl.check("gesv", tl.tl_gesv_batched(h, n, A, LU, b, x2, piv, info, layout, ld, batch), h)
+            F = A.clone()
+            tl.check("getrf", tl.tl_getrf_batched(h, n, F, layout, ld, piv, info, batch), h)
+            out.append([t.cpu().numpy().view(np.int32) for t in (x, x2, LU, F.reshape(-1)[:0] if layout else F, piv, info)])
+        tl.tl_dispatch_set(h, n, layout, 0, 0)
+        for a, c in zip(*out):
+            assert np.array_equal(a, c), (n, batch, layout)
