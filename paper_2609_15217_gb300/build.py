@@ -58,7 +58,7 @@ SPILL_ALLOW = [
     (r"k_factor_groupILi23ELi8E", 16, 16),
     # the calls of the exact general path, out of line
     (r"slow_factor_thread|slow_ragged_thread|k_getrs_thread|k_factor_threadILi[678]E|k_ragged_threadILi[89]E", 64, 64),
-    (r"k_ragged_irILi1[34]ELi4E", 64, 64),
+    (r"k_ragged_irILi(1[34]ELi4|24ELi8|32ELi16)E", 64, 64),
     # shared-memory solvers: ptxas parks a few addresses of the load and
     # store phases on the stack (the same with a higher register limit);
     # the refinement warp kernel at 64 registers (8 blocks per SM, measured

@@ -225,6 +225,7 @@ __device__ __forceinline__ bool any_nonfinite32(const float (&y)[dev::Group<N, T
 template <int N, int T>
 __global__ void __launch_bounds__(128) k_ragged_ir(RaggedArgs r)
 {
+    grid_trigger();
     constexpr int K = dev::Group<N, T>::K;
     constexpr int G = 32 / T;
     const int lane = threadIdx.x & 31;
@@ -372,6 +373,7 @@ __global__ void __launch_bounds__(128) k_ragged_ir(RaggedArgs r)
             }
         }
     }
+    if (blockIdx.x == 0) grid_wait_previous();
 }
 
 }  // namespace tl

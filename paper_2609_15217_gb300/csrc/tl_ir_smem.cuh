@@ -66,6 +66,7 @@ __device__ __forceinline__ bool any_nonfinite(float y, bool row_lane)
 template <int N>
 __global__ void __launch_bounds__(128, 8) k_smem_ir(RaggedArgs r, int)
 {
+    grid_trigger();
     constexpr int R32 = ir_row_stride32(N);
     constexpr int TC = 4, TR = 8;  // lane tile
     extern __shared__ float smem32[];
@@ -223,6 +224,7 @@ __global__ void __launch_bounds__(128, 8) k_smem_ir(RaggedArgs r, int)
         }
         __syncwarp();
     }
+    if (blockIdx.x == 0) grid_wait_previous();
 }
 
 }  // namespace tl

@@ -49,6 +49,13 @@ __device__ __forceinline__ void cp_async_wait_all()
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;\n" ::: "memory");
 }
 
+// Programmatic stream serialization: let the next kernel of the stream start
+// once every block of this grid has started (trigger), and wait for the
+// grid before this one to have completed with its memory visible (no effect
+// in a plain launch).
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void grid_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ceil(2^20 / c): floor(x / c) == (x * magic20(c)) >> 20 for 0 <= x < 1024
 // and 1 <= c <= 32 (the error x (m - 2^20/c) / 2^20 stays below 1/c).
 __host__ __device__ constexpr unsigned magic20(int c) { return (1048576u + static_cast<unsigned>(c) - 1u) / c; }

@@ -252,3 +252,41 @@ def test_ragged_autotune_table(tl):
         check_ir(systems, b_off, p_off, x, piv, info, ref)
     finally:
         tl.tl_destroy(hd)
+
+
+def test_overlapped_refinement_kernels_captured(tl, h):
+    """The refinement kernels of the sizes overlap on the stream: what follows
+    the call on the same stream sees every result, directly and from a
+    captured graph replayed over new inputs."""
+    batch = 3000
+    sizes = inputs.rng(881).integers(1, 33, size=batch).astype(np.int64)
+    d = lambda a, dt: torch.from_numpy(np.ascontiguousarray(a)).to(device=DEV, dtype=dt)  # noqa: E731
+    systems, a_off, b_off, p_off, Abuf, bbuf, npiv = make_ragged(sizes, 882)
+    dn, da, db, dp = d(sizes, torch.int32), d(a_off, torch.int64), d(b_off, torch.int64), d(p_off, torch.int64)
+    dA, dbv = d(Abuf, torch.float64), d(bbuf, torch.float64)
+    dx = torch.empty_like(dbv)
+    dpiv = torch.empty(npiv, dtype=torch.int32, device=DEV)
+    dinfo, dref = (torch.empty(batch, dtype=torch.int32, device=DEV) for _ in range(2))
+    out = [torch.empty_like(t) for t in (dx, dpiv, dinfo, dref)]
+
+    def call():
+        for t in (dx, dpiv, dinfo, dref):
+            t.fill_(-7)
+        tl.check("ragged", tl.tl_lupp_solve_batched(h, batch, dn, da, dA, db, dbv, dx, dp, dpiv, dinfo, prec=1,
+                                                    refine_steps=dref), h)
+        for o, t in zip(out, (dx, dpiv, dinfo, dref)):
+            o.copy_(t)
+
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        call()
+    torch.cuda.synchronize()
+    check_ir(systems, b_off, p_off, *(o.cpu().numpy() for o in out))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call()
+    dA.mul_(3.0)
+    dbv.mul_(0.75)
+    graph.replay()
+    torch.cuda.synchronize()
+    check_ir({n: (idx, A * 3.0, b * 0.75) for n, (idx, A, b) in systems.items()}, b_off, p_off, *(o.cpu().numpy() for o in out))
