@@ -98,9 +98,10 @@ NEWTON_GROUP_FAMILIES = [(n, t) for n, t in KERNEL_FAMILIES if n >= 10]
 # (fixed-size and ragged, with the single persistent launch), the entry
 # without allocation, the dispatcher and the peak probe.  The register
 # kernels, mixed precision, Newton and the server are not in it.
-CHECKED_SOURCES = ["tl_api.cu", "tl_inst_smem.cu", "tl_ragged.cu", "tl_noalloc.cu", "tl_autotune.cu", "tl_peak.cu"]
+CHECKED_SOURCES = ["tl_api.cu", "tl_inst_smem.cu", "tl_ragged.cu", "tl_noalloc.cu", "tl_autotune.cu", "tl_peak.cu",
+                   "tl_getrs.cu"]
 
-PLAIN_SOURCES = ["tl_api.cu", "tl_newton.cu", "tl_newton_cpu_driven.cu", "tl_ragged.cu", "tl_noalloc.cu", "tl_inst_smem.cu", "tl_autotune.cu", "tl_server.cu", "tl_newton_smem.cu", "tl_peak.cu"]
+PLAIN_SOURCES = ["tl_api.cu", "tl_newton.cu", "tl_newton_cpu_driven.cu", "tl_ragged.cu", "tl_noalloc.cu", "tl_inst_smem.cu", "tl_autotune.cu", "tl_server.cu", "tl_newton_smem.cu", "tl_peak.cu", "tl_getrs.cu"]
 
 
 def _nvcc():

@@ -402,6 +402,8 @@ tl_status tl_getrs_batched(tl_handle *h, int n, int nrhs, const double *LU, cons
     if (!ipiv || misaligned(ipiv, 4)) return fail_arg(h, 5);
     if (!B || misaligned(B, 8)) return fail_arg(h, 8);
     SolveArgs a{LU, nullptr, nullptr, B, const_cast<int32_t *>(ipiv), nullptr, ld_batch, batch, nrhs};
+    if (!h->choice[n][layout][kOpGetrs].lanes && getrs_in_shared(h, n, nrhs, layout, batch))
+        return launch_getrs_shared(h, n, layout, a, stream);
     return launch_op(h, n, layout, kOpGetrs, a, stream);
 }
 

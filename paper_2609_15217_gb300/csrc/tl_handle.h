@@ -38,6 +38,10 @@ tl_status fail_cuda(tl_handle *h, cudaError_t e);
 int pick_block(tl_handle *h, const void *kernel, int64_t threads, int lanes, size_t smem_per_system,
                int smem_limit);
 tl_status launch_variant(tl_handle *h, const Variant *v, int n, int block, SolveArgs &args, cudaStream_t stream);
+// tl_getrs with the factors in shared memory: whether it is the default, and
+// the launch.
+bool getrs_in_shared(const tl_handle *h, int n, int nrhs, int layout, int64_t batch);
+tl_status launch_getrs_shared(tl_handle *h, int n, int layout, SolveArgs &args, cudaStream_t stream);
 tl_status smem_opt_in(tl_handle *h, const void *kernel, int *limit);
 int blocks_per_sm(tl_handle *h, const void *kernel, int block, size_t smem);
 // Default ragged variant id for n: register kernels up to n = 16, the
