@@ -49,7 +49,7 @@ SPILL_ALLOW = [
     # fused Newton kernels: the law's fields, the Jacobian and the register
     # LUpp of a point live across the iteration (255 registers); measured
     # faster than the shared-memory Newton kernel up to n = 24 all the same
-    (r"k_newton_norton", 2048, 2048),
+    (r"slow_tangent", 64, 64),
     (r"k_newton_tanh", 512, 512),
     (r"slow_tanh_solve", 256, 256),
     # LU-output register variants (getrf, gesv + factors) keep L in

@@ -54,7 +54,15 @@ const void *tanh_thread_kernel(int n)
 tl_status newton_launch(tl_handle *h, int law_id, int n, const NewtonBatch &B, cudaStream_t stream)
 {
     if (B.total == 0) return TL_OK;
-    if (law_id == TL_LAW_NORTON) return launch_persistent(h, reinterpret_cast<const void *>(&k_newton_norton), 1, B, stream);
+    if (law_id == TL_LAW_NORTON) {
+        const tl_status st = launch_persistent(h, reinterpret_cast<const void *>(&k_newton_norton), 1, B, stream);
+        if (st != TL_OK || B.jobs || !B.one.tangent) return st;
+        const int64_t grid = (B.total + 127) / 128;
+        if (grid > INT32_MAX) return TL_ERR_UNSUPPORTED;
+        k_norton_tangent<<<static_cast<unsigned>(grid), 128, 0, stream>>>(B.one);
+        const cudaError_t e = cudaGetLastError();
+        return e == cudaSuccess ? TL_OK : fail_cuda(h, e);
+    }
     if (law_id != TL_LAW_TANH || n < 1 || n > TL_MAX_N) return TL_ERR_UNSUPPORTED;
     if (n <= kTanhThreadMaxN) return launch_persistent(h, tanh_thread_kernel(n), 1, B, stream);
     tl_status st = TL_OK;

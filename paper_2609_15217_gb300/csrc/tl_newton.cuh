@@ -84,39 +84,90 @@ static __device__ __noinline__ Solve7 slow_norton_solve(NortonParams P, NortonSt
     return out;
 }
 
-// Consistent tangent at a converged state (Sec. 4.3: one multi-RHS solve
-// after convergence): J X = [I_6; 0] with the six right-hand sides carried
-// through one elimination, then dsig/ddeps = C X[0..5] (Mandel elasticity
-// C = lambda 1 (x) 1 + 2 mu I).  Stores tangent[(i + 6 j) np + p]; NaN when
-// the Jacobian is singular or not finite.  Out of line: it runs once per
-// point and must not weigh on the Newton loop's registers.
-static __device__ __noinline__ void norton_tangent_store(NortonParams P, NortonState st, double *tangent, int64_t np,
-                                                         int64_t p)
+// The Jacobian at one converged point.
+__device__ __forceinline__ void tangent_jacobian(const NewtonJob &jb, int64_t p, double (&J)[7][7])
 {
-    double F[7], J[7][7], sig[6], X[6][7];
-    norton_eval(P, st.sig0, st.deps, st.x, F, J, sig);
-    const bool bad = dev::any_nonfinite<7>(J);
+    const int64_t np = jb.npoints;
+    double sig[6], x[7], n[6], pw_m;
 #pragma unroll
-    for (int c = 0; c < 6; ++c)
+    for (int i = 0; i < 7; ++i) x[i] = jb.x[i * np + p];
+    if (jb.out) {
 #pragma unroll
-        for (int i = 0; i < 7; ++i) X[c][i] = (i == c) ? 1.0 : 0.0;
-    int piv[7];
-    double rcp[7];
-    bool tiny = false;
-    const int info = dev::lu_thread_factor<7, false, 6>(J, X, piv, rcp, tiny);
+        for (int i = 0; i < 6; ++i) sig[i] = jb.out[i * np + p];
+    } else {
+        double sig0[6];
 #pragma unroll
-    for (int c = 0; c < 6; ++c) dev::lu_thread_backsolve<7>(J, X[c], rcp, tiny);
-    const bool ok = info == 0 && !bad;
-    const double two_mu = 2.0 * P.mu;
-#pragma unroll
+        for (int i = 0; i < 6; ++i) sig0[i] = jb.in[i * np + p];
+        norton_stress(jb.P, sig0, x, sig);
+    }
+    norton_jacobian(jb.P, sig, x[6], n, pw_m, J);
+}
+
+// Solve for the six columns with the factors of J (L as stored by LAPACK) and
+// store the tangent.
+template <bool FAST>
+__device__ __forceinline__ void tangent_columns(const NewtonJob &jb, int64_t p, const double (&J)[7][7],
+                                                const int (&piv)[7], const double (&rcp)[7], bool tiny, bool ok)
+{
+#pragma unroll 1
     for (int j = 0; j < 6; ++j) {
-        const double tr = X[j][0] + X[j][1] + X[j][2];
+        double y[7];
+#pragma unroll
+        for (int i = 0; i < 7; ++i) y[i] = i == j ? 1.0 : 0.0;
+        dev::lu_thread_forward<7>(J, piv, y);
+        if (FAST) dev::lu_thread_backsolve_fast<7>(J, y, rcp);
+        else dev::lu_thread_backsolve<7>(J, y, rcp, tiny);
+        const double tr = y[0] + y[1] + y[2];
 #pragma unroll
         for (int i = 0; i < 6; ++i) {
-            const double d = (i < 3) ? fma(P.lambda, tr, two_mu * X[j][i]) : two_mu * X[j][i];
-            tangent[(i + 6 * j) * np + p] = ok ? d : dev::nan_value();
+            const double d = (i < 3) ? fma(jb.P.lambda, tr, jb.P.two_mu * y[i]) : jb.P.two_mu * y[i];
+            st_stream(jb.tangent + (i + 6 * j) * jb.npoints + p, ok ? d : dev::nan_value());
         }
     }
+}
+
+// The exact general path of one point (a zero, tiny, huge or non-finite pivot).
+static __device__ __noinline__ void slow_tangent(const NewtonJob &jb, int64_t p)
+{
+    double J[7][7], none[1][7], rcp[7];
+    int piv[7];
+    bool tiny = false;
+    tangent_jacobian(jb, p, J);
+    const bool bad = dev::any_nonfinite<7>(J);
+    const int info = dev::lu_thread_factor<7, true, 0>(J, none, piv, rcp, tiny);
+    dev::lu_thread_unnegate_L<7>(J);
+    tangent_columns<false>(jb, p, J, piv, rcp, tiny, info == 0 && !bad);
+}
+
+// Consistent tangent at the converged states (Sec. 4.3: one multi-RHS solve
+// after convergence): J X = [I_6; 0] with one factorization, then dsig/ddeps
+// = C X[0..5] (Mandel elasticity C = lambda 1 (x) 1 + 2 mu I).  Stores tangent[(i + 6 j) np + p]; NaN when
+// the point did not converge or the Jacobian is singular or not finite.
+// J depends on the stress and on dp alone; the stress is the one stored in
+// `out`, or formed from sig0 and x where the caller keeps none.
+// A launch of its own after k_newton_norton, one thread per point: inside the
+// Newton loop a warp ran these 570 FP64 instructions in almost every trip
+// for the few lanes that had just converged (400,000 points: 2421 us in all
+// that way, 1960 us with this launch and the law's shorter evaluation).
+static __global__ void __launch_bounds__(128) k_norton_tangent(const __grid_constant__ NewtonJob jb)
+{
+    const int64_t p = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int64_t np = jb.npoints;
+    if (p >= np) return;
+    if (jb.status[p] != TL_NEWTON_CONVERGED) {
+        for (int i = 0; i < 36; ++i) jb.tangent[i * np + p] = dev::nan_value();
+        return;
+    }
+    double J[7][7], none[1][7], rcp[7];
+    int piv[7];
+    tangent_jacobian(jb, p, J);
+    const bool bad = dev::any_nonfinite<7>(J);
+    if (dev::lu_thread_factor_fast<7, true, 0, true>(J, none, piv, rcp) || bad) {
+        slow_tangent(jb, p);
+        return;
+    }
+    dev::lu_thread_unnegate_L<7>(J);
+    tangent_columns<true>(jb, p, J, piv, rcp, false, true);
 }
 
 static __global__ void __launch_bounds__(128) k_newton_norton(NewtonBatch B)
@@ -187,21 +238,6 @@ static __global__ void __launch_bounds__(128) k_newton_norton(NewtonBatch B)
         if (jb.out) {
 #pragma unroll
             for (int i = 0; i < 6; ++i) jb.out[i * np + p] = sig[i];
-        }
-        if (jb.tangent) {
-            if (st == TL_NEWTON_CONVERGED) {
-                NortonState ns;
-#pragma unroll
-                for (int i = 0; i < 6; ++i) {
-                    ns.sig0[i] = sig0[i];
-                    ns.deps[i] = deps[i];
-                }
-#pragma unroll
-                for (int i = 0; i < 7; ++i) ns.x[i] = x[i];
-                norton_tangent_store(P, ns, jb.tangent, np, p);
-            } else {
-                for (int i = 0; i < 36; ++i) jb.tangent[i * np + p] = dev::nan_value();
-            }
         }
         jb.iters[p] = k;
         jb.status[p] = st;
@@ -398,7 +434,7 @@ __global__ void __launch_bounds__(128) k_newton_tanh_group(NewtonBatch B)
         }
 #pragma unroll
         for (int off = T / 2; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-        const double r = sqrt(ss);
+        const double r = dev::sqrt_rn(ss);
         if (have && fresh) r0 = r;
         fresh = false;
         int st = have ? newton_decide<N>(r, r0, k, B.rtol, B.max_iter) : 0;

@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) k_newton_tanh_smem(Newton
         }
 #pragma unroll
         for (int off = T / 2; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-        const double r = sqrt(ss);
+        const double r = dev::sqrt_rn(ss);
         if (have && fresh) r0 = r;
         fresh = false;
         int st = have ? newton_decide<32>(r, r0, k, B.rtol, B.max_iter) : 0;
