@@ -6,9 +6,8 @@
 // (F_i = sum_j a_ij x_j + c_i tanh(x_i) - b_i with the sum as fma in
 // increasing j; J = A + diag(c .* (1 - tanh^2 x))) into the augmented block
 // [J | -F], the warp factors every group's block and solves for dx, and
-// the group updates x.  ||F||_2: each lane's fma sum over its rows, then a
-// butterfly over the group.  Persistent: a group whose point stops stores
-// it and takes the next one of its stride.
+// the group updates x.  Persistent: a group whose point stops stores it and
+// takes the next one of its stride.
 #include <cmath>
 
 #include "tinylu.h"
@@ -20,33 +19,49 @@
 namespace tl {
 namespace {
 
-// Warps per block: 2 keeps 14 instead of 12 warps resident at n = 19..20
-// (+6%); within +-2% of 1 and 4 warps elsewhere (measured at n = 10..32).
+// Warps per block: within 3% of 1 and 4 (measured at n = 10..32), and no
+// size is left without room for a block.
 constexpr int kWarpsPerBlock = 2;
 
 // Lanes per point of the shared-memory kernel for the tanh law at size n;
 // 0 where the sub-warp register kernel runs (n = 10; n <= 9 runs one
-// thread per point).  Measured on GB300 (points/s over n = 10..32 for
-// every lane count and the register kernels): 4 lanes win at n = 11..14,
-// 8 at 15..22, 16 at 23..28, 32 from 29; 9-56% over the register kernels.
-int newton_smem_lanes(int n)
+// thread per point).  Measured on GB300 (million points/s, 131,072 or 65,536
+// points): n = 13: 4 lanes 65.3, 8 lanes 62.3; n = 18: 41.6, 42.7; n = 23:
+// 8 lanes 25.0, 16 lanes 22.1; n = 25: 18.6, 18.4; n = 29: 11.5, 13.2; 32 lanes
+// never for so many (n = 32: 9.8 against 10.6 with 16).  While there are few
+// points a wider group shortens each of their steps, as in the fixed-size
+// solves; a point's results are the same with any lane count.
+int newton_smem_lanes(const tl_handle *h, int n, int64_t points)
 {
     if (n <= 10 || n > TL_MAX_N) return 0;
-    if (n <= 14) return 4;
-    if (n <= 22) return 8;
-    if (n <= 28) return 16;
-    return 32;
+    const int lanes = n <= 14 ? 4 : n <= 25 ? 8 : 16;
+    for (int T : {32, 16, 8})
+        if (T > lanes && points * T <= 32 * 16 * h->sm_count) return T;
+    return lanes;
 }
 
 // Shared memory per point: the solver's block plus 32 doubles of x.
 __host__ __device__ constexpr int newton_smem_doubles(int n, int T) { return smem_sys_doubles(n, T) + 32; }
 
-// T lanes per point, 32 / T points per warp.  Every trip of the loop each
-// group with a live point assembles [J | -F] of its point (lane t the rows
-// t, t + T, ...), the warp factors every group's block with the shared-
-// memory solver (warp-synchronous, so groups without a point factor a
-// stale block and ignore it), and each group updates x, decides, and on a
-// stop stores the point and takes the next one of its stride.
+// Whether |v| is infinite or NaN, on its high word.
+__device__ __forceinline__ bool high_nonfinite(double v)
+{
+    return (static_cast<unsigned>(__double2hiint(v)) & 0x7ff00000u) == 0x7ff00000u;
+}
+
+// T lanes per point, 32 / T points per warp.  In every trip of the loop each
+// group with a live point factors and solves its system [J | -F] (the warp
+// together; groups without a point factor a stale block and ignore it),
+// updates x, assembles the next system at the new x and decides; a group whose
+// point stops stores it and takes the next one of its stride before the next
+// trip, so no solve is idle while points are left.  At the first guess x = 0
+// the system is A + diag(c) and -F = b: no products and no tanh are needed, so a
+// new point costs copies (and the look for non-finite entries, whose products
+// with 0 would be NaN).  A is copied into the block by cp.async, all entries in
+// flight, while the lanes evaluate tanh; A x is then summed from there.
+// Measured at n = 20 with 8 lanes, 65,537 points, against one assembly per
+// trip with the entries loaded one by one and a trip without a solve at the end
+// of each point: 2214 -> 1926 us.
 template <int T>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock) k_newton_tanh_smem(NewtonBatch B, int n)
 {
@@ -65,69 +80,125 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) k_newton_tanh_smem(Newton
     int64_t np = 1, p = 0;
     double r0 = 0.0;
     int k = 0;
-    bool fresh = true;
-    while (__any_sync(0xffffffffu, have)) {
-        if (have && fresh) {
-            const NewtonJob jb = load_job(B, g);
-            in = jb.in;
-            np = jb.npoints;
-            p = g - jb.start;
-            for (int i = t; i < n; i += T) xs[i] = 0.0;
-            k = 0;
+
+    // copy this lane's rows of A into the block
+    auto copy_rows = [&]() {
+        for (int i = t; i < n; i += T) {
+            const double *src = in + static_cast<int64_t>(i) * np + p;
+            const int64_t step = static_cast<int64_t>(n) * np;
+            for (int j = 0; j < n; ++j, src += step) cp_async8(M + i * RS + j, src);
+        }
+    };
+    // ||F||_2 from the squares of the lane's rows, by the same tree over 32
+    // rows whatever T is (rows i and i + 16, then + 8, ...), so that a point's
+    // decisions do not depend on the lanes that its launch gives it
+    auto group_norm = [&](double (&sq)[KM]) {
+#pragma unroll
+        for (int off = 16; off >= T; off >>= 1)
+#pragma unroll
+            for (int s = 0; s < off / T; ++s) sq[s] += sq[s + off / T];
+        double ss = sq[0];
+#pragma unroll
+        for (int off = T / 2; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+        return dev::sqrt_rn(ss);
+    };
+    auto store_point = [&](int st) {
+        const NewtonJob jb = load_job(B, g);
+        for (int i = t; i < n; i += T) jb.x[i * np + p] = xs[i];
+        if (t == 0) {
+            jb.iters[p] = k;
+            jb.status[p] = st;
+        }
+        g += ngroups;
+        have = g < B.total;
+    };
+
+    bool fresh = have;
+    for (;;) {
+        // groups without an assembled system take their next point, until it
+        // needs a solve
+        while (__any_sync(0xffffffffu, fresh)) {
+            double sq[KM] = {};
+            if (fresh) {
+                const NewtonJob jb = load_job(B, g);
+                in = jb.in;
+                np = jb.npoints;
+                p = g - jb.start;
+                k = 0;
+                copy_rows();
+                cp_async_wait_all();
+#pragma unroll
+                for (int s = 0; s < KM; ++s) {
+                    const int i = t + s * T;
+                    if (i >= n) break;
+                    xs[i] = 0.0;
+                    const double ci = in[(n * n + i) * np + p];
+                    const double bi = in[(n * n + n + i) * np + p];
+                    bool bad = high_nonfinite(ci);
+                    for (int j = 0; j < n; ++j) bad = bad || high_nonfinite(M[i * RS + j]);
+                    M[i * RS + i] = __dadd_rn(M[i * RS + i], ci);
+                    const double Fi = bad ? dev::nan_value() : 0.0 - bi;
+                    M[i * RS + n] = dev::neg(Fi);
+                    sq[s] = Fi * Fi;
+                }
+            }
+            const double r = group_norm(sq);
+            if (fresh) {
+                r0 = r;
+                const int st = newton_decide<32>(r, r0, 0, B.rtol, B.max_iter);
+                if (st >= 0) store_point(st);
+                fresh = st >= 0 && have;
+            }
         }
         __syncwarp();
-        // assemble this lane's rows of [J | -F]
-        double ss = 0.0;
+        if (!__any_sync(0xffffffffu, have)) break;
+        // solve and update
+        unsigned worst;  // a non-finite Jacobian shows in the next residual
+        const int info = smem_lupp2<T, true, false>(M, n, RS, t, 0, 0.0, worst);
+        int st = -1;
+        if (have) {
+            if (info != 0) {
+                st = TL_NEWTON_SINGULAR;
+            } else {
+                for (int i = t; i < n; i += T) xs[i] += M[i * RS + n];
+                ++k;
+            }
+        }
+        __syncwarp();
+        // the system at the new x
+        const bool go = have && st < 0;
+        double sq[KM] = {};
+        if (go) copy_rows();
+        double ti[KM];
 #pragma unroll
         for (int s = 0; s < KM; ++s) {
             const int i = t + s * T;
-            if (have && i < n) {
-                const double xi = xs[i];
-                const double ti = tanh(xi);
+            ti[s] = 0.0;
+            if (go && i < n) ti[s] = tanh(xs[i]);
+        }
+        cp_async_wait_all();
+#pragma unroll
+        for (int s = 0; s < KM; ++s) {
+            const int i = t + s * T;
+            if (go && i < n) {
                 const double ci = in[(n * n + i) * np + p];
                 const double bi = in[(n * n + n + i) * np + p];
                 double acc = 0.0;
-                for (int j = 0; j < n; ++j) {
-                    const double aij = in[(j * n + i) * np + p];
-                    acc = fma(aij, xs[j], acc);
-                    M[i * RS + j] = (j == i) ? fma(ci, fma(-ti, ti, 1.0), aij) : aij;
-                }
-                const double Fi = fma(ci, ti, acc) - bi;
+#pragma unroll 4
+                for (int j = 0; j < n; ++j) acc = fma(M[i * RS + j], xs[j], acc);
+                M[i * RS + i] = fma(ci, fma(-ti[s], ti[s], 1.0), M[i * RS + i]);
+                const double Fi = fma(ci, ti[s], acc) - bi;
                 M[i * RS + n] = dev::neg(Fi);
-                ss = fma(Fi, Fi, ss);
+                sq[s] = Fi * Fi;
             }
         }
-#pragma unroll
-        for (int off = T / 2; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-        const double r = dev::sqrt_rn(ss);
-        if (have && fresh) r0 = r;
+        const double r = group_norm(sq);
+        if (go) st = newton_decide<32>(r, r0, k, B.rtol, B.max_iter);
+        __syncwarp();
         fresh = false;
-        int st = have ? newton_decide<32>(r, r0, k, B.rtol, B.max_iter) : 0;
-        const bool need = have && st < 0;
-        __syncwarp();
-        if (__any_sync(0xffffffffu, need)) {
-            unsigned worst;  // a non-finite Jacobian shows in the next residual
-            const int info = smem_lupp2<T, true, false>(M, n, RS, t, 0, 0.0, worst);
-            if (need) {
-                if (info != 0) {
-                    st = TL_NEWTON_SINGULAR;
-                } else {
-                    for (int i = t; i < n; i += T) xs[i] += M[i * RS + n];
-                    ++k;
-                }
-            }
-        }
-        __syncwarp();
         if (have && st >= 0) {
-            const NewtonJob jb = load_job(B, g);
-            for (int i = t; i < n; i += T) jb.x[i * np + p] = xs[i];
-            if (t == 0) {
-                jb.iters[p] = k;
-                jb.status[p] = st;
-            }
-            g += ngroups;
-            have = g < B.total;
-            fresh = true;
+            store_point(st);
+            fresh = have;
         }
     }
 }
@@ -159,7 +230,7 @@ tl_status launch_smem_newton(tl_handle *h, int n, const NewtonBatch &B, cudaStre
 // for the others).
 bool newton_tanh_smem_launch(tl_handle *h, int n, const NewtonBatch &B, cudaStream_t stream, tl_status *out)
 {
-    switch (newton_smem_lanes(n)) {
+    switch (newton_smem_lanes(h, n, B.total)) {
     case 4: *out = launch_smem_newton<4>(h, n, B, stream); return true;
     case 8: *out = launch_smem_newton<8>(h, n, B, stream); return true;
     case 16: *out = launch_smem_newton<16>(h, n, B, stream); return true;

@@ -215,3 +215,31 @@ def test_norton_tangent_parity(tl, h):
         tl.TL_ERR_UNSUPPORTED
     assert tl.tl_newton_integrate_tangent(h, law, 4, d_in, d_x, None, None, d_it, d_st, 1e-10, 20) == \
         tl.TL_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("n,npts", [(11, 9729), (14, 9728), (15, 4865), (20, 4864), (25, 4865), (26, 2433), (32, 2433)])
+def test_tanh_lanes_do_not_matter(tl, h, n, npts):
+    """Points on both sides of the lines where the lanes per point change
+    with their number (152 SMs): every point's state, iteration count and
+    status bit for bit as in a call with a few points, with points that stop
+    at once or do not converge among them."""
+    A, c, b = inputs.tanh_points(n, npts, 5100 + n)
+    A[5, 1, 1] = np.nan
+    A[9] = 0.0
+    c[9] = 0.0                      # singular
+    b[13] = 0.0                     # converged at the first guess
+    c[17, 0] = np.inf
+    def run(sel):
+        k = len(sel)
+        f = np.concatenate([A[sel].transpose(0, 2, 1).reshape(k, n * n).T, c[sel].T, b[sel].T])
+        d = torch.from_numpy(np.ascontiguousarray(f)).cuda()
+        x = torch.zeros((n, k), dtype=torch.float64, device="cuda")
+        it, st = (torch.zeros(k, dtype=torch.int32, device="cuda") for _ in range(2))
+        tl.check("newton", tl.tl_newton_integrate(h, tl.make_law(tl.TL_LAW_TANH, n), k, d, x, None, it, st, 1e-10, 20), h)
+        return x.cpu().numpy(), it.cpu().numpy(), st.cpu().numpy()
+    x, it, st = run(np.arange(npts))
+    for sel in (np.arange(40), np.arange(npts - 700, npts)):
+        xs, its, sts = run(sel)
+        assert np.array_equal(xs.view(np.int64), x[:, sel].copy().view(np.int64))
+        assert np.array_equal(its, it[sel]) and np.array_equal(sts, st[sel])
+    assert st[5] == st[17] == tl.TL_NEWTON_NONFINITE and st[9] == tl.TL_NEWTON_SINGULAR and (st[13], it[13]) == (0, 0)
