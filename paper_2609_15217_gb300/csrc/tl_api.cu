@@ -226,6 +226,7 @@ tl_status launch_variant(tl_handle *h, const Variant *v, int n, int block, Solve
     const size_t smem = (block / v->lanes) * per_sys;
     if (smem > static_cast<size_t>(dyn_limit)) return TL_ERR_UNSUPPORTED;
     if (shared) {
+        args.ahead = static_cast<int64_t>(std::max(1, blocks_per_sm(h, v->kernel, block, smem))) * h->sm_count;
         int nn = n;
         void *params[] = {&args, &nn};
         e = cudaLaunchKernel(v->kernel, dim3(static_cast<unsigned>(grid)), dim3(block), params, smem, stream);

@@ -26,6 +26,8 @@ struct SolveArgs {
     // tile-local pivoting (shared-memory kernels only): 0 = textbook
     int tile;
     double threshold;
+    // blocks of the launch that are resident at once (set by launch_variant)
+    int64_t ahead;
 };
 
 // Arguments of the ragged-batch kernels (tl_lupp_solve_batched): the

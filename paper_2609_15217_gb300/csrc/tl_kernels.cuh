@@ -49,6 +49,9 @@ __device__ __forceinline__ void cp_async_wait_all()
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;\n" ::: "memory");
 }
 
+// Fetch the line at p into L2.
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // Programmatic stream serialization: let the next kernel of the stream start
 // once every block of this grid has started (trigger), and wait for the
 // grid before this one to have completed with its memory visible (no effect
