@@ -845,26 +845,30 @@ __global__ void __launch_bounds__(128) k_smem_group(SolveArgs args, int n)
     if constexpr (KEEP) {
         // the factors by the mapping of the loads (a group's own entries of
         // one column lie in as many rows of the interleaved storage: 50,000
-        // systems of n = 13 145 us that way, 139 us now); the slot of the first
+        // systems of n = 13 145 us that way, 131 us now); the slot of the first
         // reciprocal tells the block whether the system had bad input
         if (t == 0) M[smem_rcp_offset(n)] = bad ? 1.0 : 0.0;
         __syncthreads();
-        auto store = [&](const double *Mq, int e, int64_t ai) {
-            const int j = div20(e, m20), i = e - j * n;
-            const double v = Mq[i * RS + j];
-            if (Mq[smem_rcp_offset(n)] == 0.0) st_stream(args.LU + ai, j < i ? dev::neg(v) : v);
-            else if (MODE == kGesv) args.LU[ai] = args.A[ai];  // nothing is factored: A
+        // entries e0, e0 + step, ... of system qs, entry e at LU[e * es + base]
+        auto store = [&](int qs, int e0, int step, int64_t base, int64_t es) {
+            const double *Mq = smem + qs * per;
+            if (Mq[smem_rcp_offset(n)] == 0.0) {
+#pragma unroll 4
+                for (int e = e0; e < nn; e += step) {
+                    const int j = div20(e, m20), i = e - j * n;
+                    const double v = Mq[i * RS + j];
+                    st_stream(args.LU + (base + e * es), j < i ? dev::neg(v) : v);
+                }
+            } else if (MODE == kGesv) {  // nothing is factored: A
+                for (int e = e0; e < nn; e += step) args.LU[base + e * es] = args.A[base + e * es];
+            }
         };
         if (LAYOUT == kInterleaved) {
-            const int qs = threadIdx.x % SB, tp = threadIdx.x / SB;
-            if (s0 + qs < args.batch) {
-#pragma unroll 4
-                for (int e = tp; e < nn; e += T) store(smem + qs * per, e, static_cast<int64_t>(e) * args.ld + s0 + qs);
-            }
+            const int qs = threadIdx.x % SB;
+            if (s0 + qs < args.batch) store(qs, threadIdx.x / SB, T, s0 + qs, args.ld);
         } else {
             for (int qs = threadIdx.x >> 5; qs < SB && s0 + qs < args.batch; qs += blockDim.x >> 5)
-#pragma unroll 4
-                for (int e = lane; e < nn; e += 32) store(smem + qs * per, e, (s0 + qs) * nn + e);
+                store(qs, lane, 32, (s0 + qs) * nn, 1);
         }
     }
 }
