@@ -82,18 +82,18 @@ int default_ragged_id(int n)
 // n = 17: 4 lanes 0.89, 8 lanes 0.87; n = 18: 0.85, 0.88; n = 24: 8 lanes
 // 0.85, 16 lanes 0.81; n = 25: 0.82, 0.86; 32 lanes never (n = 32: 0.82
 // against 0.87).  Per system 8 lanes already win at n = 17 (0.92 against
-// 0.90) and up to n = 26 (0.90, 0.90).  With the factors stored the next lane
-// count wins earlier, and 32 lanes from n = 27 on (interleaved, 0.745 against
-// 0.707) or n = 31 (per system, 0.868 against 0.860).
+// 0.90) and up to n = 26 (0.90, 0.90).  With the factors stored, gesv:
+// interleaved n = 16 4 lanes 0.81, 8 lanes 0.79; n = 18 0.78, 0.82; n = 22 8
+// lanes 0.79, 16 lanes 0.77; n = 23 0.79, 0.80; per system n = 14 0.84, 0.79;
+// n = 15 0.80, 0.83; n = 23 0.89, 0.84; n = 25 0.84, 0.87.
 int default_lanes(int n, int layout, int op)
 {
     const bool inter = layout == TL_LAYOUT_INTERLEAVED;
     if (n <= 9) return variant_id(1, 0);
     if (op == kOpGesvLU || op == kOpGetrf) {
-        if (n <= 10) return variant_id(2, 2);
-        if (n <= 14) return variant_id(4, 2);
-        if (n <= (inter ? 24 : 22)) return variant_id(8, 2);
-        return n <= (inter ? 26 : 30) ? variant_id(16, 1) : variant_id(32, 1);
+        if (n <= 10 && op == kOpGesvLU) return variant_id(2, 2);
+        if (n <= (inter ? 17 : 14)) return variant_id(4, 2);
+        return n <= (inter ? 22 : 23) ? variant_id(8, 2) : variant_id(16, 1);
     }
     if (n <= 10) return variant_id(2, 2);
     if (n <= (inter ? 17 : 16)) return variant_id(4, 2);
@@ -107,12 +107,13 @@ int default_lanes(int n, int layout, int op)
 // Interleaved, a block of b threads reads 8 b / lanes consecutive bytes of
 // each entry: 64 threads for up to 8 lanes (n = 19: 0.87, with 128 threads
 // 0.85), 128 above (n = 30: 0.89, with 64 0.86); one warp is enough for 2
-// and 4 lanes (n = 13: 0.89, 64 threads 0.88), also when the batch would
-// otherwise leave SMs without a block.
-int default_block(tl_handle *h, const Variant *v, int layout, int64_t batch)
+// lanes, and for 4 unless the factors are stored (n = 13: 0.89, 64 threads
+// 0.88; with the factors 0.81, 0.82), also when the batch would otherwise
+// leave SMs without a block.
+int default_block(tl_handle *h, const Variant *v, int layout, int op, int64_t batch)
 {
     if (v->kind == 0) return 0;
-    if (layout == TL_LAYOUT_PER_SYSTEM || v->lanes <= 4) return 32;
+    if (layout == TL_LAYOUT_PER_SYSTEM || v->lanes <= (op == kOpGesv ? 4 : 2)) return 32;
     const int block = v->lanes <= 8 ? 64 : 128;
     return batch * v->lanes < static_cast<int64_t>(block) * h->sm_count ? 32 : block;
 }
@@ -283,7 +284,7 @@ tl_status launch_op(tl_handle *h, int n, int layout, int op, SolveArgs &args, cu
     }
     const Variant *v = find_variant(n, layout, op, c.lanes ? c.lanes : default_lanes(n, layout, op));
     if (!v) return TL_ERR_UNSUPPORTED;
-    return launch_variant(h, v, n, c.lanes ? c.block : default_block(h, v, layout, args.batch), args, stream);
+    return launch_variant(h, v, n, c.lanes ? c.block : default_block(h, v, layout, op, args.batch), args, stream);
 }
 
 static bool misaligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) != 0; }

@@ -27,7 +27,7 @@ struct PairHash {
 };
 
 int default_lanes(int n, int layout, int op);
-int default_block(tl_handle *h, const Variant *v, int layout, int64_t batch);
+int default_block(tl_handle *h, const Variant *v, int layout, int op, int64_t batch);
 int default_register_lanes(int n);
 // Default mixed-precision ragged variant id for n: one thread, then 4 lanes
 // per system in registers, then the shared-memory warp kernel.
