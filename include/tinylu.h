@@ -317,6 +317,9 @@ tl_status tl_newton_integrate(tl_handle *h, const tl_law *law, int64_t npoints,
  *   tangent  device double[36 * npoints]:
  *            tangent[(i + 6 j) * npoints + p] = dsig_i / ddeps_j; NaN for
  *            points that did not converge.
+ * Runs as a second launch after the Newton loop (it reads x, the status and
+ * the stress in outputs, or sig0 when outputs is NULL, so outputs may overwrite
+ * sig0 in place).
  * Other arguments as tl_newton_integrate (tangent is argument 7; the
  * arguments after it are numbered one higher).  TL_LAW_TANH returns
  * TL_ERR_UNSUPPORTED.
@@ -398,7 +401,8 @@ tl_status tl_autotune_ragged(tl_handle *h, int n_min, int n_max, const char *tab
 
 /*
  * tl_ragged_dispatch_set / tl_ragged_dispatch_get -- per size n: lanes per
- * system of the persistent ragged launch (0 = default: one thread with the
+ * system of the persistent ragged launch (0 = default, wider for batches of a
+ * few thousand systems; otherwise one thread with the
  * system in registers up to n = 7, then 2 lanes up to n = 10, 4 up to 14, 8 up
  * to 22, 16 above; 1 (n <= 7 only) or 2..32 a power of two) and the
  * mixed-precision route (-1 = default: refine from n = 21 on, binary64
@@ -419,13 +423,15 @@ tl_status tl_ragged_dispatch_get(tl_handle *h, int n, int *lanes, int *refines);
  *            n, n >= 2; 2..32 lanes; the trailing update of 2..8 lanes on a
  *            lane tile, of 16 and 32 lanes element by element), 2 = shared
  *            memory with the element-by-element trailing update for 2..8
- *            lanes.  0 restores the built-in default.  A
- *            variant not built for n is rejected with TL_ERR_INVALID_ARG
- *            (argument 4).
+ *            lanes.  0 restores the built-in default, which for small
+ *            batches runs wider groups than the variant that get returns.
+ *            A variant not built for n is rejected with
+ *            TL_ERR_INVALID_ARG (argument 4).
  *   block    0 (occupancy + wave-fill heuristic) or 32, 64, 128 threads.
  * The choice applies to tl_gesv_batched and tl_getrf_batched for (n,
  * layout); tl_getrs_batched uses the register kernel with the same lane
- * count when one exists; the two parts of tl_lupp_solve_batched take the
+ * count when one exists (else its default, which depends on n, nrhs, the
+ * layout and the batch); the two parts of tl_lupp_solve_batched take the
  * register or shared-memory ragged kernel of the same id when one exists.
  * Their defaults: binary64, register kernels up to n = 16, shared memory
  * with 16 lanes up to n = 26, 32 lanes above; mixed precision, one thread
