@@ -65,7 +65,9 @@ __device__ __forceinline__ void getrs_load(const SolveArgs &args, int n, int64_t
     for (int e = tid; e < live * n; e += nth) {
         const int q = LAYOUT == kInterleaved ? e % live : e / n, k = LAYOUT == kInterleaved ? e / live : e % n;
         int *row = reinterpret_cast<int *>(smem + q * per + n * RS + n);
-        row[k] = args.ipiv[LAYOUT == kInterleaved ? static_cast<int64_t>(k) * args.ld + s0 + q : (s0 + q) * n + k] - 1;
+        const int p =
+            args.ipiv[LAYOUT == kInterleaved ? static_cast<int64_t>(k) * args.ld + s0 + q : (s0 + q) * n + k] - 1;
+        row[k] = p > k && p < n ? p : k;  // what getrf never writes is no interchange (row indexes memory)
     }
     cp_async_wait_all();
     __syncthreads();
