@@ -46,9 +46,8 @@ CHECK_FLAGS = ["-DTL_CHECK_BOUNDS=1"]
 # may use: (regex on the mangled name, max store bytes, max load bytes).
 # Every other kernel must not spill at all.
 SPILL_ALLOW = [
-    # fused Newton kernels: the law's fields, the Jacobian and the register
-    # LUpp of a point live across the iteration (255 registers); measured
-    # faster than the shared-memory Newton kernel up to n = 24 all the same
+    # the exact general path of the tangent, out of line; the tanh-law
+    # kernels with the Jacobian and the register LUpp of a point in registers
     (r"slow_tangent", 64, 64),
     (r"k_newton_tanh", 512, 512),
     (r"slow_tanh_solve", 256, 256),
