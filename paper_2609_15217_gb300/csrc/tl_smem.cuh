@@ -537,9 +537,12 @@ __device__ __forceinline__ void smem_multipliers(double *M, int n, int RS, int k
 
 // Returns info; worst receives the largest high word of the magnitudes of
 // A's entries and of the values that replaced them, as this lane met them: a
-// non-finite entry of A stays non-finite until it is in a pivot column or in
-// a row of U, so only when some lane of the group reports 0x7ff00000 or more
-// can A hold one.
+// non-finite entry of A stays non-finite until it is the pivot or in a row of
+// U, or, below a smaller pivot that is not zero, until its multiplier has
+// spread along its row.  A zero pivot above such an entry, which tile-local
+// pivoting with a threshold of 0 keeps, spreads it nowhere: a system with a
+// zero pivot reports 0x7ff00000 there.  So only when some lane of the group
+// reports 0x7ff00000 or more can A hold a non-finite entry.
 template <int T, bool SOLVE, bool KEEPL>
 __device__ __forceinline__ int smem_lupp2(double *M, int n, int RS, int t, int tile, double threshold, unsigned &worst)
 {
@@ -651,6 +654,8 @@ __device__ __forceinline__ int smem_lupp2(double *M, int n, int RS, int t, int t
         tiny = tiny || s0;
         __syncwarp();
     }
+
+    if (tile > 0 && info != 0) worst = 0x7ff00000u;
 
     // a6 (back part): x_i = y_i * RN(1/u_ii) (y_i / u_ii when a pivot was
     // below DBL_MIN), then y_r -= u_ri x_i for r < i

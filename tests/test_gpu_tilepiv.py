@@ -29,12 +29,12 @@ def h(tl):
     tl.tl_destroy(hh)
 
 
-def run(tl, h, A, b, tile, layout, thr=1e-10):
+def run(tl, h, A, b, tile, layout, thr=1e-10, want_lu=True):
     batch, n = A.shape[0], A.shape[1]
     ld = L.pad_ld(batch)
     dA = L.matrices_to_layout(torch.from_numpy(A).to(DEV), layout, ld)
     db = L.vectors_to_layout(torch.from_numpy(b).to(DEV), layout, ld)
-    dLU = torch.empty_like(dA)
+    dLU = torch.empty_like(dA) if want_lu else None
     dx = torch.empty_like(db)
     dpiv = torch.empty(db.numel(), dtype=torch.int32, device=DEV)
     dinfo = torch.empty(batch, dtype=torch.int32, device=DEV)
@@ -42,7 +42,7 @@ def run(tl, h, A, b, tile, layout, thr=1e-10):
     torch.cuda.synchronize()
     return (L.vectors_from_layout(dx, batch, n, layout, ld).cpu().numpy(),
             L.vectors_from_layout(dpiv, batch, n, layout, ld).cpu().numpy(), dinfo.cpu().numpy(),
-            L.matrices_from_layout(dLU, batch, n, layout, ld).cpu().numpy())
+            L.matrices_from_layout(dLU, batch, n, layout, ld).cpu().numpy() if want_lu else None)
 
 
 @pytest.mark.parametrize("n", [2, 5, 9, 12, 17, 32])
@@ -75,6 +75,38 @@ def test_tile_zero_is_textbook(tl, h):
     for tile in (0, n, 40):
         x, piv, info, LU = run(tl, h, A, b, tile, 1)
         assert np.array_equal(piv, piv_o) and np.array_equal(LU.view(np.int64), LU_o.view(np.int64))
+
+
+@pytest.mark.parametrize("layout", [0, 1], ids=["per_system", "interleaved"])
+@pytest.mark.parametrize("n", [5, 12, 20, 21, 32])
+def test_nonfinite_entry_below_a_zero_tile(tl, h, n, layout):
+    """Threshold 0: a step whose tile holds only zeros keeps its zero pivot,
+    so a NaN or Inf below the tile in that column spreads to no other entry.
+    info = -1 all the same (identity pivots, LU_out = A, x = NaN)."""
+    tile = 4 if n > 5 else 2
+    steps = [0, 1, tile - 1, tile, n - 3, n - 2]
+    A, b = inputs.uniform_systems(n, 4 * len(steps) + 3, 7300 + n)
+    planted = 0
+    for q, k in enumerate(steps):
+        end = min(n, (k // tile + 1) * tile)
+        if end == n:
+            continue
+        for w, (row, v) in enumerate(((end, np.nan), (n - 1, np.inf), (n - 1, -np.inf), (end, 0.0))):
+            # column k of the rows up to the tile's end stays exactly zero
+            A[4 * q + w, :end, k] = 0.0
+            A[4 * q + w, row, k] = v
+            planted += not np.isfinite(v)
+    LU_o, piv_o, info_o, _ = oracle.getrf_tiled(A, tile, 0.0)
+    assert (info_o == -1).sum() == planted > 0 and (info_o > 0).any()
+    for want_lu in (True, False):
+        x, piv, info, LU = run(tl, h, A, b, tile, layout, 0.0, want_lu)
+        assert np.array_equal(info, info_o)
+        assert np.array_equal(piv, piv_o)
+        assert np.isnan(x[info_o != 0]).all()
+        if want_lu:
+            good = info_o >= 0
+            assert np.array_equal(LU[good].view(np.int64), LU_o[good].view(np.int64))
+            assert np.array_equal(LU[~good], A[~good], equal_nan=True)
 
 
 def test_tilepiv_argument_errors(tl, h):
