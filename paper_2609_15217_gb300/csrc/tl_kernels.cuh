@@ -355,6 +355,9 @@ __global__ void __launch_bounds__(128) k_getrs_group(SolveArgs args)
         rcp[sl] = dev::rcp_rn(d);
         tiny = tiny || (ok && dev::mag_bits(d) < dev::kDblMinBits);
     }
+    // one pivot below DBL_MIN: quotients for every row of the system, as in
+    // the other solves
+    tiny = group_any<T>(tiny);
     for (int r = 0; r < args.nrhs; ++r) {
         double y[K];
 #pragma unroll
