@@ -317,9 +317,10 @@ tl_status tl_newton_integrate(tl_handle *h, const tl_law *law, int64_t npoints,
  *   tangent  device double[36 * npoints]:
  *            tangent[(i + 6 j) * npoints + p] = dsig_i / ddeps_j; NaN for
  *            points that did not converge.
- * Runs as a second launch after the Newton loop (it reads x, the status and
- * the stress in outputs, or sig0 when outputs is NULL, so outputs may overwrite
- * sig0 in place).
+ * Runs as a second launch after the Newton loop.  It reads what that one
+ * stored, not the inputs, so x or outputs may overwrite the inputs in place;
+ * with outputs NULL the first six rows of tangent carry the stress between
+ * the two launches.
  * Other arguments as tl_newton_integrate (tangent is argument 7; the
  * arguments after it are numbered one higher).  TL_LAW_TANH returns
  * TL_ERR_UNSUPPORTED.

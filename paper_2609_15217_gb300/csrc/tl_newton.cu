@@ -55,11 +55,14 @@ tl_status newton_launch(tl_handle *h, int law_id, int n, const NewtonBatch &B, c
 {
     if (B.total == 0) return TL_OK;
     if (law_id == TL_LAW_NORTON) {
-        const tl_status st = launch_persistent(h, reinterpret_cast<const void *>(&k_newton_norton), 1, B, stream);
-        if (st != TL_OK || B.jobs || !B.one.tangent) return st;
+        NewtonBatch N = B;
+        const bool tangent = !B.jobs && B.one.tangent;
+        if (tangent && !N.one.out) N.one.out = N.one.tangent;  // see k_norton_tangent
+        const tl_status st = launch_persistent(h, reinterpret_cast<const void *>(&k_newton_norton), 1, N, stream);
+        if (st != TL_OK || !tangent) return st;
         const int64_t grid = (B.total + 127) / 128;
         if (grid > INT32_MAX) return TL_ERR_UNSUPPORTED;
-        k_norton_tangent<<<static_cast<unsigned>(grid), 128, 0, stream>>>(B.one);
+        k_norton_tangent<<<static_cast<unsigned>(grid), 128, 0, stream>>>(N.one);
         const cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? TL_OK : fail_cuda(h, e);
     }

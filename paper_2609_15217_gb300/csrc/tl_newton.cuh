@@ -84,23 +84,15 @@ static __device__ __noinline__ Solve7 slow_norton_solve(NortonParams P, NortonSt
     return out;
 }
 
-// The Jacobian at one converged point.
+// The Jacobian at one converged point: a function of the stress that the
+// Newton launch stored in `out` and of dp.
 __device__ __forceinline__ void tangent_jacobian(const NewtonJob &jb, int64_t p, double (&J)[7][7])
 {
     const int64_t np = jb.npoints;
-    double sig[6], x[7], n[6], pw_m;
+    double sig[6], n[6], pw_m;
 #pragma unroll
-    for (int i = 0; i < 7; ++i) x[i] = jb.x[i * np + p];
-    if (jb.out) {
-#pragma unroll
-        for (int i = 0; i < 6; ++i) sig[i] = jb.out[i * np + p];
-    } else {
-        double sig0[6];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) sig0[i] = jb.in[i * np + p];
-        norton_stress(jb.P, sig0, x, sig);
-    }
-    norton_jacobian(jb.P, sig, x[6], n, pw_m, J);
+    for (int i = 0; i < 6; ++i) sig[i] = jb.out[i * np + p];
+    norton_jacobian(jb.P, sig, jb.x[6 * np + p], n, pw_m, J);
 }
 
 // Solve for the six columns with the factors of J (L as stored by LAPACK) and
@@ -143,8 +135,10 @@ static __device__ __noinline__ void slow_tangent(const NewtonJob &jb, int64_t p)
 // after convergence): J X = [I_6; 0] with one factorization, then dsig/ddeps
 // = C X[0..5] (Mandel elasticity C = lambda 1 (x) 1 + 2 mu I).  Stores tangent[(i + 6 j) np + p]; NaN when
 // the point did not converge or the Jacobian is singular or not finite.
-// J depends on the stress and on dp alone; the stress is the one stored in
-// `out`, or formed from sig0 and x where the caller keeps none.
+// J depends on the stress and on dp alone, so the inputs, which x may have
+// overwritten, are not read again: where the caller keeps no stress, `out` is
+// the first six rows of `tangent` (a thread reads its point's before it
+// stores the tangent over them).
 // A launch of its own after k_newton_norton, one thread per point: inside the
 // Newton loop a warp ran these 570 FP64 instructions in almost every trip
 // for the few lanes that had just converged (400,000 points: 2421 us in all

@@ -179,6 +179,26 @@ def test_newton_argument_errors(tl, h):
     assert tl.tl_newton_integrate(h, law, 4, d, d, None, i, i, 1e-10, 20) == tl.TL_ERR_INVALID_ARG
 
 
+def test_norton_tangent_with_the_state_over_the_inputs(tl, h):
+    """x written over the input fields (each point reads its fields before it
+    stores), with and without the stress: the tangent of separate arrays."""
+    npts = 700
+    sig0, deps = inputs.norton_points(npts, 57)
+    law = tl.make_law(tl.TL_LAW_NORTON, 7, oracle.norton_params())
+    out = []
+    for alias, want_sig in ((False, True), (True, True), (True, False)):
+        d_in = torch.from_numpy(np.ascontiguousarray(np.concatenate([sig0.T, deps.T], axis=0))).to(DEV)
+        d_x = d_in[:7] if alias else torch.empty((7, npts), dtype=torch.float64, device=DEV)
+        d_sig = torch.empty((6, npts), dtype=torch.float64, device=DEV) if want_sig else None
+        d_D = torch.empty((36, npts), dtype=torch.float64, device=DEV)
+        d_it, d_st = (torch.empty(npts, dtype=torch.int32, device=DEV) for _ in range(2))
+        tl.check("tangent", tl.tl_newton_integrate_tangent(h, law, npts, d_in, d_x, d_sig, d_D, d_it, d_st, 1e-10, 20), h)
+        assert (d_st == 0).all()
+        out.append((d_x.cpu().numpy(), d_D.cpu().numpy()))
+    for x, D in out[1:]:
+        assert np.array_equal(x, out[0][0]) and np.array_equal(D, out[0][1])
+
+
 def test_norton_tangent_parity(tl, h):
     """Consistent tangent (Sec. 4.3, multi-RHS solve after convergence)
     against the oracle's, point by point; states and counts unchanged."""
