@@ -48,13 +48,17 @@ constexpr float kRefineMargin = 0.85f;
 // each other changed from one bench run to the next; 4 narrow that noise.
 constexpr int kTuneReps = 5;
 
-// The choice of tl_gesv_batched / tl_getrf_batched for (n, layout), and for
-// tl_getrs_batched the register kernel with the same lane count when there
-// is one.  The ragged solves keep their own table (tl_autotune_ragged).
+// The choice of tl_gesv_batched / tl_getrf_batched for (n, layout).
 void set_gesv_family(tl_handle *h, int n, int layout, int variant, int block)
 {
     for (int op = 0; op < kOps; ++op)
         if (op_takes_variant(op)) h->choice[n][layout][op] = Choice{variant, block};
+}
+
+// For tl_getrs_batched the register kernel with the same lane count when
+// there is one.
+void set_getrs(tl_handle *h, int n, int layout, int variant)
+{
     const int lanes = variant % 100;
     const VariantList &lo = registry(n, layout, kOpGetrs);
     for (int i = 0; i < lo.count; ++i)
@@ -108,6 +112,7 @@ extern "C" tl_status tl_dispatch_set(tl_handle *h, int n, tl_layout layout, int 
         if (l.v[i].kind != kKindLatency && variant_id(l.v[i].lanes, l.v[i].kind) == variant) found = true;
     if (!found) return fail_arg(h, 4);
     set_gesv_family(h, n, layout, variant, block);
+    set_getrs(h, n, layout, variant);
     // the ragged kernels (binary64 and mixed precision): the register kernel
     // with the same lane count, or the shared-memory kernel of the same id,
     // when there is one
@@ -236,7 +241,11 @@ extern "C" tl_status tl_autotune(tl_handle *h, int n_min, int n_max, tl_layout l
             }
         }
         if (st == TL_OK && best_var) {
+            // tl_getrs_batched was not timed: its own rule by n, nrhs, layout and
+            // batch stays (n = 27, 178,062 systems, six right-hand sides:
+            // 2272 us, the register kernel of the same lanes 3781)
             set_gesv_family(h, n, layout, best_var, best_block);
+            h->choice[n][layout][kOpGetrs] = Choice{0, 0};
             table.push_back(Row{n, best_var, best_block, best_ms});
         }
     }

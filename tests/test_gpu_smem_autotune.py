@@ -5,6 +5,7 @@ convention).  Same bar as the register kernels: pivots, info and LU
 bit-identical to the oracle, x within BE 10 n and FE 1e-12 kappa."""
 import json
 import os
+import re
 import tempfile
 
 import numpy as np
@@ -131,3 +132,44 @@ def test_autotune_table_and_parity(tl, h):
         x_g, piv_g, info_g, _ = gpu_gesv(tl, h, A, b, 1, want_lu=False)
         assert np.array_equal(piv_g, piv_o) and np.array_equal(info_g, info_o)
         check_solution(A, b, x_g, x_o)
+
+
+def kernels_launched(call):
+    """Names of the kernels that a call launches (from a capture of it)."""
+    call()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    g.enable_debug_mode()
+    with torch.cuda.graph(g):
+        call()
+    path = os.path.join(tempfile.mkdtemp(), "call.dot")
+    g.debug_dump(path)
+    names = re.findall(r"k_[a-z][A-Za-z0-9_]*", open(path).read())
+    assert names
+    return sorted(set(names))
+
+
+@pytest.mark.parametrize("layout", [0, 1], ids=["per_system", "interleaved"])
+@pytest.mark.parametrize("n", [8, 27])
+@pytest.mark.parametrize("call", ["getrs"])
+@pytest.mark.filterwarnings("ignore:DEBUG")
+def test_tuning_keeps_what_it_does_not_measure(tl, h, call, n, layout):
+    """tl_autotune times tl_gesv_batched on large batches: solves with given
+    factors launch the kernels of an untuned handle.  A variant set with
+    tl_dispatch_set holds for them too."""
+    from paper_2609_15217_gb300 import layout as L
+    batch = 64
+    ld = L.pad_ld(batch)
+    A = L.matrices_to_layout(torch.eye(n, dtype=torch.float64, device=DEV).repeat(batch, 1, 1), layout, ld)
+    B = L.multi_rhs_to_layout(torch.ones((batch, 6, n), dtype=torch.float64, device=DEV), layout, ld)
+    piv = torch.arange(1, n + 1, dtype=torch.int32, device=DEV).repeat(batch, 1)
+    piv = L.vectors_to_layout(piv, layout, ld)
+
+    def run():
+        tl.check("getrs", tl.tl_getrs_batched(h, n, 6, A, piv, layout, ld, B, batch), h)
+
+    untuned = kernels_launched(run)
+    assert tl.tl_autotune(h, n, n, layout, None) == tl.TL_OK
+    assert kernels_launched(run) == untuned
+    assert tl.tl_dispatch_set(h, n, layout, 1 if n <= 9 else 16, 0) == tl.TL_OK
+    assert kernels_launched(run) != untuned
