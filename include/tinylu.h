@@ -357,7 +357,9 @@ tl_status tl_newton_integrate_cpu_driven(tl_handle *h, const tl_law *law, int64_
  * "best X" size-aware dispatcher, Sec. 4.1) for tl_gesv_batched and
  * tl_getrf_batched; tl_getrs_batched, which is not timed, returns to its
  * built-in choice, and the ragged solves keep their own table
- * (tl_autotune_ragged).  table_path nullable: if given, the table is
+ * (tl_autotune_ragged).  The timed batches are large: small batches keep the
+ * wider groups of the built-in default (a variant set with tl_dispatch_set
+ * holds for every batch).  table_path nullable: if given, the table is
  * also written there as JSON.  Allocates and frees a temporary device batch;
  * must not run during stream capture.
  */
@@ -395,7 +397,8 @@ tl_status tl_measure_fma_peak(tl_handle *h, int bits, double *tflops, double *fm
  * tuning batch: systems whose conditioning defeats the refinement fall back
  * to binary64 and pay for both, so workloads with many such systems may
  * prefer binary64 for more sizes).
- * The choices stay in the handle; table_path (nullable) receives them as
+ * The choices stay in the handle (batches of a few thousand systems still
+ * take wider groups, as by default); table_path (nullable) receives them as
  * JSON.  Allocates and frees a temporary device batch; synchronizes; must
  * not run during stream capture.
  */

@@ -239,7 +239,8 @@ tl_status launch_variant(tl_handle *h, const Variant *v, int n, int block, Solve
     return TL_OK;
 }
 
-// Variant and block of a small batch (null: the large-batch default).  A
+// Variant of a small batch, wider than the `lanes` of a large one (null: as a
+// large batch).  A
 // warp alone on a sub-partition runs at the pace of its own FP64
 // instructions and of each step's latency, so while a wider group still
 // leaves every sub-partition few warps, it is faster: fewer FP64 instructions
@@ -251,10 +252,9 @@ tl_status launch_variant(tl_handle *h, const Variant *v, int n, int block, Solve
 // these: 64 systems of n = 6 7.2 -> 4.5 us; 4,096 of n = 8 14.2 -> 6.8; 1,024
 // of n = 16 35.4 -> 14.9; 256 of n = 20 36 -> 16.5; 4,096 of n = 32 154 ->
 // 127.
-static const Variant *small_batch_variant(tl_handle *h, int n, int layout, int op, int64_t batch)
+static const Variant *small_batch_variant(tl_handle *h, int n, int layout, int op, int lanes, int64_t batch)
 {
     const int64_t sms = h->sm_count;
-    const int id0 = default_lanes(n, layout, op);
     if (n <= 16) {
         const VariantList &l = registry(n, layout, op);
         for (int i = 0; i < l.count; ++i) {
@@ -268,7 +268,7 @@ static const Variant *small_batch_variant(tl_handle *h, int n, int layout, int o
     }
     if (n < 10 || op == kOpGetrs) return nullptr;
     for (int T : {32, 16, 8, 4}) {
-        if (T <= id0 % 100) break;
+        if (T <= lanes) break;
         if (batch * T <= 32 * 16 * sms || (T == 32 && n >= 28 && batch <= 8192))
             return find_variant(n, layout, op, variant_id(T, T >= 16 ? 1 : 2));
     }
@@ -278,11 +278,12 @@ static const Variant *small_batch_variant(tl_handle *h, int n, int layout, int o
 tl_status launch_op(tl_handle *h, int n, int layout, int op, SolveArgs &args, cudaStream_t stream)
 {
     const Choice &c = h->choice[n][layout][op];
-    if (!c.lanes) {
-        const Variant *small = small_batch_variant(h, n, layout, op, args.batch);
+    const int id = c.lanes ? c.lanes : default_lanes(n, layout, op);
+    if (!c.lanes || c.tuned) {
+        const Variant *small = small_batch_variant(h, n, layout, op, id % 100, args.batch);
         if (small) return launch_variant(h, small, n, 32, args, stream);
     }
-    const Variant *v = find_variant(n, layout, op, c.lanes ? c.lanes : default_lanes(n, layout, op));
+    const Variant *v = find_variant(n, layout, op, id);
     if (!v) return TL_ERR_UNSUPPORTED;
     return launch_variant(h, v, n, c.lanes ? c.block : default_block(h, v, layout, op, args.batch), args, stream);
 }

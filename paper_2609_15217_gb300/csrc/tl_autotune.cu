@@ -49,10 +49,10 @@ constexpr float kRefineMargin = 0.85f;
 constexpr int kTuneReps = 5;
 
 // The choice of tl_gesv_batched / tl_getrf_batched for (n, layout).
-void set_gesv_family(tl_handle *h, int n, int layout, int variant, int block)
+void set_gesv_family(tl_handle *h, int n, int layout, int variant, int block, bool tuned)
 {
     for (int op = 0; op < kOps; ++op)
-        if (op_takes_variant(op)) h->choice[n][layout][op] = Choice{variant, block};
+        if (op_takes_variant(op)) h->choice[n][layout][op] = Choice{variant, block, tuned};
 }
 
 // For tl_getrs_batched the register kernel with the same lane count when
@@ -111,7 +111,7 @@ extern "C" tl_status tl_dispatch_set(tl_handle *h, int n, tl_layout layout, int 
     for (int i = 0; i < l.count; ++i)
         if (l.v[i].kind != kKindLatency && variant_id(l.v[i].lanes, l.v[i].kind) == variant) found = true;
     if (!found) return fail_arg(h, 4);
-    set_gesv_family(h, n, layout, variant, block);
+    set_gesv_family(h, n, layout, variant, block, false);
     set_getrs(h, n, layout, variant);
     // the ragged kernels (binary64 and mixed precision): the register kernel
     // with the same lane count, or the shared-memory kernel of the same id,
@@ -244,7 +244,7 @@ extern "C" tl_status tl_autotune(tl_handle *h, int n_min, int n_max, tl_layout l
             // tl_getrs_batched was not timed: its own rule by n, nrhs, layout and
             // batch stays (n = 27, 178,062 systems, six right-hand sides:
             // 2272 us, the register kernel of the same lanes 3781)
-            set_gesv_family(h, n, layout, best_var, best_block);
+            set_gesv_family(h, n, layout, best_var, best_block, true);
             h->choice[n][layout][kOpGetrs] = Choice{0, 0};
             table.push_back(Row{n, best_var, best_block, best_ms});
         }
@@ -411,7 +411,7 @@ extern "C" tl_status tl_autotune_ragged(tl_handle *h, int n_min, int n_max, cons
     cleanup();
     if (st != TL_OK) return st;
     for (const Row &row : table) {
-        if (row.lanes) h->choice[row.n][kPerSystem][kOpRagged] = Choice{variant_id(row.lanes, 1), 0};
+        if (row.lanes) h->choice[row.n][kPerSystem][kOpRagged] = Choice{variant_id(row.lanes, 1), 0, true};
         if (row.ir_variant) h->choice[row.n][kPerSystem][kOpRaggedIr] = Choice{row.ir_variant, 0};
         h->mixed_route[row.n] = static_cast<signed char>(row.refine ? 0 : 1);
     }

@@ -14,9 +14,12 @@ namespace tl {
 
 // Dispatch choice for one (n, layout, op): lanes per system (0 = default
 // policy) and block size (0 = occupancy + wave-fill heuristic per launch).
+// `tuned`: found by a tuner, whose batches are large; the rules of small
+// batches stay in force.
 struct Choice {
     int lanes;
     int block;
+    bool tuned = false;
 };
 
 struct PairHash {

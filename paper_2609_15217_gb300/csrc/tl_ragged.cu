@@ -179,13 +179,13 @@ bool mixed_refines(const tl_handle *h, int n)
 int persist_lanes(const tl_handle *h, int n, int limit, int64_t batch)
 {
     int T = default_persist_lanes(n);
-    const int id = h->choice[n][kPerSystem][kOpRagged].lanes;
+    const Choice &c = h->choice[n][kPerSystem][kOpRagged];
     bool chosen = false;
-    if (id >= 100) {
-        const int L = id % 100;
+    if (c.lanes >= 100) {
+        const int L = c.lanes % 100;
         if ((L == 1 && n <= kPersistRegMaxN) || L == 2 || L == 4 || L == 8 || L == 16 || L == 32) {
             T = L;
-            chosen = true;
+            chosen = !c.tuned;
         }
     }
     // a batch that gives each sub-partition few warps: wider groups, as in the

@@ -151,12 +151,12 @@ def kernels_launched(call):
 
 @pytest.mark.parametrize("layout", [0, 1], ids=["per_system", "interleaved"])
 @pytest.mark.parametrize("n", [8, 27])
-@pytest.mark.parametrize("call", ["getrs"])
+@pytest.mark.parametrize("call", ["gesv", "getrs"])
 @pytest.mark.filterwarnings("ignore:DEBUG")
 def test_tuning_keeps_what_it_does_not_measure(tl, h, call, n, layout):
-    """tl_autotune times tl_gesv_batched on large batches: solves with given
-    factors launch the kernels of an untuned handle.  A variant set with
-    tl_dispatch_set holds for them too."""
+    """tl_autotune times tl_gesv_batched on large batches: small ones, and
+    solves with given factors, launch the kernels of an untuned handle.  A
+    variant set with tl_dispatch_set holds for them too."""
     from paper_2609_15217_gb300 import layout as L
     batch = 64
     ld = L.pad_ld(batch)
@@ -165,7 +165,12 @@ def test_tuning_keeps_what_it_does_not_measure(tl, h, call, n, layout):
     piv = torch.arange(1, n + 1, dtype=torch.int32, device=DEV).repeat(batch, 1)
     piv = L.vectors_to_layout(piv, layout, ld)
 
+    info = torch.zeros(batch, dtype=torch.int32, device=DEV)
+    piv2, x = torch.zeros_like(piv), torch.zeros(piv.numel(), dtype=torch.float64, device=DEV)
+
     def run():
+        if call == "gesv":
+            return tl.check("gesv", tl.tl_gesv_batched(h, n, A, None, B, x, piv2, info, layout, ld, batch), h)
         tl.check("getrs", tl.tl_getrs_batched(h, n, 6, A, piv, layout, ld, B, batch), h)
 
     untuned = kernels_launched(run)
