@@ -246,8 +246,8 @@ tl_status launch_variant(tl_handle *h, const Variant *v, int n, int block, Solve
 // leaves every sub-partition few warps, it is faster: fewer FP64 instructions
 // and shorter passes per warp.  n = 5..16 with one row per lane in registers
 // (8 lanes up to n = 8, else 16) up to 12 or 8 warps per SM; the element walk
-// with 32, 16, 8 or 4 lanes up to 16 warps per SM (32 lanes up to 8,192
-// systems from n = 28 on, where a wider group costs least).  Measured per call
+// with 32, 16, 8 or 4 lanes up to 16 warps per SM (32 lanes up to 54 systems
+// per SM from n = 28 on, where a wider group costs least).  Measured per call
 // in a CUDA graph, one thread per system or the large-batch lanes against
 // these: 64 systems of n = 6 7.2 -> 4.5 us; 4,096 of n = 8 14.2 -> 6.8; 1,024
 // of n = 16 35.4 -> 14.9; 256 of n = 20 36 -> 16.5; 4,096 of n = 32 154 ->
@@ -269,7 +269,7 @@ static const Variant *small_batch_variant(tl_handle *h, int n, int layout, int o
     if (n < 10 || op == kOpGetrs) return nullptr;
     for (int T : {32, 16, 8, 4}) {
         if (T <= lanes) break;
-        if (batch * T <= 32 * 16 * sms || (T == 32 && n >= 28 && batch <= 8192))
+        if (batch * T <= 32 * 16 * sms || (T == 32 && n >= 28 && batch <= 54 * sms))
             return find_variant(n, layout, op, variant_id(T, T >= 16 ? 1 : 2));
     }
     return nullptr;
@@ -308,6 +308,10 @@ tl_status tl_create(tl_handle **out)
         e = cudaDeviceGetAttribute(&h->max_threads_per_sm, cudaDevAttrMaxThreadsPerMultiProcessor, h->device);
     if (e == cudaSuccess)
         e = cudaDeviceGetAttribute(&h->max_smem_per_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&h->smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, h->device);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&h->smem_reserved, cudaDevAttrReservedSharedMemoryPerBlock, h->device);
     if (e != cudaSuccess) {
         delete h;
         return TL_ERR_CUDA;
@@ -405,8 +409,10 @@ tl_status tl_getrs_batched(tl_handle *h, int n, int nrhs, const double *LU, cons
     if (!ipiv || misaligned(ipiv, 4)) return fail_arg(h, 5);
     if (!B || misaligned(B, 8)) return fail_arg(h, 8);
     SolveArgs a{LU, nullptr, nullptr, B, const_cast<int32_t *>(ipiv), nullptr, ld_batch, batch, nrhs};
-    if (!h->choice[n][layout][kOpGetrs].lanes && getrs_in_shared(h, n, nrhs, layout, batch))
-        return launch_getrs_shared(h, n, layout, a, stream);
+    if (!h->choice[n][layout][kOpGetrs].lanes && getrs_in_shared(h, n, nrhs, layout, batch)) {
+        const tl_status st = launch_getrs_shared(h, n, layout, a, stream);
+        if (st != TL_ERR_UNSUPPORTED) return st;
+    }
     return launch_op(h, n, layout, kOpGetrs, a, stream);
 }
 

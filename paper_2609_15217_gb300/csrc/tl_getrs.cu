@@ -1,7 +1,5 @@
 // tl_getrs.cu -- launches of the shared-memory solves with given factors
 // (tl_getrs.cuh).
-#include <algorithm>
-
 #include "tl_getrs.cuh"
 #include "tl_handle.h"
 
@@ -59,39 +57,16 @@ tl_status launch_getrs_shared(tl_handle *h, int n, int layout, SolveArgs &args, 
     int limit = 0;
     const tl_status st = smem_opt_in(h, kern, &limit);
     if (st != TL_OK) return st;
-    int SB = 1, block = 32;
-    size_t smem = 0;
-    if (rows) {
-        block = 64;
-        SB = block / 8;
-        smem = static_cast<size_t>(getrs_block_doubles(n, SB)) * 8;
-    } else {
-        // systems per block: the most useful lanes per SM, up to the two
-        // warps per sub-partition that keep the FP64 pipe busy
-        double best = -1.0;
-        const int most = std::min<int64_t>(128 / args.nrhs, args.batch);
-        for (int sb = 1; sb <= most; ++sb) {
-            const int threads = (sb * args.nrhs + 31) / 32 * 32;
-            const size_t bytes = (static_cast<size_t>(getrs_block_doubles(n, sb)) + static_cast<size_t>(n) * threads) * 8;
-            if (bytes > static_cast<size_t>(limit)) break;
-            const int blocks = static_cast<int>(233472 / (bytes + 1024));
-            const int warps = std::min(8, blocks * threads / 32);
-            const double score = warps * static_cast<double>(sb * args.nrhs) / threads;
-            if (score >= best) {
-                best = score;
-                SB = sb;
-                block = threads;
-                smem = bytes;
-            }
-        }
-        if (best < 0.0) return TL_ERR_UNSUPPORTED;
-    }
-    const int64_t grid = (args.batch + SB - 1) / SB;
+    GetrsPlan plan{};
+    if (!(rows ? getrs_rows_plan(n, limit, &plan)
+               : getrs_rhs_plan(n, args.nrhs, args.batch, limit, h->smem_per_sm, h->smem_reserved, &plan)))
+        return TL_ERR_UNSUPPORTED;
+    const int64_t grid = (args.batch + plan.SB - 1) / plan.SB;
     if (grid > INT32_MAX) return TL_ERR_UNSUPPORTED;
     int nn = n;
-    void *params[] = {&args, &nn, &SB};
-    const cudaError_t e = cudaLaunchKernel(kern, dim3(static_cast<unsigned>(grid)), dim3(static_cast<unsigned>(block)),
-                                           params, smem, stream);
+    void *params[] = {&args, &nn, &plan.SB};
+    const cudaError_t e = cudaLaunchKernel(kern, dim3(static_cast<unsigned>(grid)),
+                                           dim3(static_cast<unsigned>(plan.block)), params, plan.smem, stream);
     return e == cudaSuccess ? TL_OK : fail_cuda(h, e);
 }
 

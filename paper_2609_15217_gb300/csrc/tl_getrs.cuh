@@ -16,18 +16,11 @@
 #pragma once
 #include "tinylu.h"
 #include "tl_bounds.cuh"
+#include "tl_getrs_plan.h"
 #include "tl_kernels.cuh"
 #include "tl_smem.cuh"
 
 namespace tl {
-
-// One system in shared memory: n rows of n entries (odd stride), n
-// reciprocals, n pivots and n source rows of P (int32); an odd number of
-// doubles, so that the systems of a warp start on distinct banks.
-__host__ __device__ constexpr int getrs_row_stride(int n) { return n | 1; }
-__host__ __device__ constexpr int getrs_sys_doubles(int n) { return (n * getrs_row_stride(n) + 2 * n) | 1; }
-// Doubles of a block of SB systems: theirs and a flag each.
-__host__ __device__ constexpr int getrs_block_doubles(int n, int SB) { return SB * getrs_sys_doubles(n) + (SB + 1) / 2; }
 
 // Copy the factors of `live` systems from s0 on into shared memory
 // (system q at q * per) and form their reciprocals and row orders.  All

@@ -42,7 +42,8 @@ int pick_block(tl_handle *h, const void *kernel, int64_t threads, int lanes, siz
                int smem_limit);
 tl_status launch_variant(tl_handle *h, const Variant *v, int n, int block, SolveArgs &args, cudaStream_t stream);
 // tl_getrs with the factors in shared memory: whether it is the default, and
-// the launch.
+// the launch (TL_ERR_UNSUPPORTED, with nothing launched, where a block does
+// not fit: the register kernels serve the call).
 bool getrs_in_shared(const tl_handle *h, int n, int nrhs, int layout, int64_t batch);
 tl_status launch_getrs_shared(tl_handle *h, int n, int layout, SolveArgs &args, cudaStream_t stream);
 tl_status smem_opt_in(tl_handle *h, const void *kernel, int *limit);
@@ -73,6 +74,8 @@ struct tl_handle {
     int sm_count = 1;
     int max_threads_per_sm = 2048;
     int max_smem_per_block = 48 * 1024;
+    int smem_per_sm = 48 * 1024;
+    int smem_reserved = 1024;  // of every resident block, on top of its own
     int last_cuda_error = 0;
     int last_bad_arg = 0;
     int ragged_mode = TL_RAGGED_PERSISTENT;  // tl_ragged_set_mode
