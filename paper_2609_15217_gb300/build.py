@@ -46,14 +46,13 @@ CHECK_FLAGS = ["-DTL_CHECK_BOUNDS=1"]
 # may use: (regex on the mangled name, max store bytes, max load bytes).
 # Every other kernel must not spill at all.
 SPILL_ALLOW = [
-    # the exact general path of the tangent, out of line; the tanh-law
-    # kernels with the Jacobian and the register LUpp of a point in registers
-    (r"slow_tangent", 64, 64),
-    (r"k_newton_tanh", 512, 512),
-    (r"slow_tanh_solve", 256, 256),
+    # the tanh-law kernel of n = 9 with the Jacobian and the register LUpp of a
+    # point in registers, and its exact general path, out of line
+    (r"k_newton_tanh", 96, 96),
+    (r"slow_tanh_solve", 128, 128),
     # LU-output register variants (getrf, gesv + factors) keep L in
     # registers as well; tuned dispatch runs the shared-memory solver there
-    (r"k_factor_groupILi\d+ELi\d+ELi\d+ELi\d+ELb1E", 640, 640),
+    (r"k_factor_groupILi\d+ELi\d+ELi\d+ELi\d+ELb1E", 256, 256),
     (r"k_factor_groupILi23ELi8E", 16, 16),
     # the calls of the exact general path, out of line
     (r"slow_factor_thread|slow_ragged_thread|k_getrs_thread|k_factor_threadILi[678]E|k_ragged_threadILi[89]E", 64, 64),
@@ -89,9 +88,9 @@ IR_FAMILIES = (
     + [(n, 16) for n in range(25, 33)]
 )
 
-# (n, lanes per point) of the sub-warp tanh-law Newton kernel (n >= 10;
-# smaller n run one thread per point).
-NEWTON_GROUP_FAMILIES = [(n, t) for n, t in KERNEL_FAMILIES if n >= 10]
+# (n, lanes per point) of the sub-warp tanh-law Newton kernel (smaller n run
+# one thread per point, larger n in shared memory).
+NEWTON_GROUP_FAMILIES = [(n, t) for n, t in KERNEL_FAMILIES if n == 10]
 
 # Units of the bounds-checked library: the C ABI, the shared-memory solvers
 # (fixed-size and ragged, with the single persistent launch), the entry

@@ -1,8 +1,9 @@
 // tl_newton.cu -- launches of the fused per-point Newton kernels of
 // tl_newton.cuh (Algorithm 2 of the paper) and the C ABI entry
 // tl_newton_integrate.  The Norton kernel and the one-thread tanh kernels
-// (n <= 9) are instantiated here; the sub-warp tanh kernels (n >= 10) come
-// from the instantiation units tl_inst_newton.cu through the registry.
+// (n <= 9) are instantiated here; the sub-warp tanh kernel (n = 10) comes
+// from the instantiation unit tl_inst_newton.cu through the registry, the
+// shared-memory one (n >= 11) from tl_newton_smem.cu.
 #include <cmath>
 
 #include "tinylu.h"

@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(128) k_newton_tanh(NewtonBatch B)
     }
 }
 
-// T lanes per point (N >= 10): lane t holds rows and unknowns t + s*T.  The
+// T lanes per point (N = 10): lane t holds rows and unknowns t + s*T.  The
 // warp runs one Newton step of each of its 32/T points per trip (a
 // warp-uniform loop, since the LUpp shuffles across the group); a group
 // whose point stops stores it and starts its next point on the next trip.

@@ -11,8 +11,8 @@
 //     element, lane t taking every T-th element row-major, and the updates
 //     of two elimination steps are applied in one pass; see its comment.
 //   * smem_lupp: one step per pass on a TR x TC tile of lanes (lane (tr, tc)
-//     keeps its columns of the pivot row in registers and walks its rows)
-//     or an element walk; kept for the lane-tile variants.
+//     keeps its columns of the pivot row in registers and walks its rows);
+//     2, 4 or 8 lanes, kept for the lane-tile variants.
 // The kernels: k_smem_group (fixed-size batches, both layouts, loads into
 // shared memory by cp.async) and k_smem_ragged (one size of a ragged batch,
 // the per-size mode).
@@ -79,18 +79,17 @@ __device__ __forceinline__ int group_any_int(int v)
 // column n holds x when SOLVE.  Returns info.  Every lane of the warp must
 // call it together (shuffles and votes inside).
 //
-// Trailing updates either walk the trailing block element by element (WALK:
-// lane t takes every T-th element, row-major) or use a TR x TC tile of
-// lanes: lane (tr, tc) updates rows k+1+tr, k+1+tr+TR, ... and columns
-// k+1+tc, k+1+tc+TC, ..., keeping its columns of the pivot row in registers.
-template <int T, bool SOLVE, bool WALK = (T >= 16)>
+// Trailing updates on a TR x TC tile of lanes: lane (tr, tc) updates rows
+// k+1+tr, k+1+tr+TR, ... and columns k+1+tc, k+1+tc+TC, ..., keeping its
+// columns of the pivot row in registers.
+template <int T, bool SOLVE>
 __device__ __forceinline__ int smem_lupp(double *M, int n, int RS, int t, int tile, double threshold)
 {
     constexpr int MODE = SOLVE ? kGesv : kGetrf;
-    constexpr int TC = WALK ? 1 : (T >= 4) ? 4 : T;  // lane tile (when not walking elements)
+    constexpr int TC = T >= 4 ? 4 : T;  // lane tile
     constexpr int TR = T / TC;
     constexpr int MAXC = TL_MAX_N / TC;  // whole column chunks per lane (at most 32 live columns)
-    static_assert(WALK || MAXC <= 16, "the chunk switch below covers 16 chunks");
+    static_assert(MAXC <= 16, "the chunk switch below covers 16 chunks");
     static_assert(T >= 1 && T <= 32 && (32 % T) == 0, "T must divide 32");
     const int tr = t / TC, tc = t % TC;
     double *rcp = M + n * RS;                              // n doubles
@@ -155,37 +154,12 @@ __device__ __forceinline__ int smem_lupp(double *M, int n, int RS, int t, int ti
         }
         __syncwarp();
         // a5 (+ forward part of a6 through column n): a_ij += (-l_ik) u_kj.
-        if (!zero && WALK) {
-            // element walk: the R x C trailing block (R = n-k-1
-            // rows, C live columns) is walked row-major, lane t taking the
-            // elements t, t+T, t+2T, ...; every lane issues ceil(R C / T)
-            // FMAs, the least any split can (a TR x TC lane tile issues
-            // ceil(R/TR) ceil(C/TC)).  l_i and u_j come from shared memory.
-            const int ncols = wcols - (k + 1);
-            const int nrows = n - (k + 1);
-            const int nel = nrows * ncols;
-            if (nel > 0) {
-                const int q = T / ncols, rq = T % ncols;  // (row, column) advance per stride
-                int ei = t / ncols, ej = t % ncols;        // element t: row k+1+ei, column k+1+ej
-                const double *urow = M + k * RS + k + 1;
-                for (int e = t; e < nel; e += T) {
-                    double *Mi = M + (k + 1 + ei) * RS;
-                    const double l = Mi[k];
-                    Mi[k + 1 + ej] = __fma_rn(l, urow[ej], Mi[k + 1 + ej]);
-                    ej += rq;
-                    ei += q;
-                    if (ej >= ncols) {
-                        ej -= ncols;
-                        ++ei;
-                    }
-                }
-            }
-        } else if (!zero) {
-            // fewer lanes: lane (tr, tc) owns columns k+1+tc + c*TC: nfull
-            // whole chunks (the same count on every lane of the warp) and
-            // possibly one tail column; the chunks are a straight-line
-            // fall-through block entered once per row, with immediate
-            // offsets from the row pointer
+        if (!zero) {
+            // lane (tr, tc) owns columns k+1+tc + c*TC: nfull whole chunks
+            // (the same count on every lane of the warp) and possibly one
+            // tail column; the chunks are a straight-line fall-through block
+            // entered once per row, with immediate offsets from the row
+            // pointer
             const int ncols = wcols - (k + 1);
             const int nfull = ncols / TC;
             const bool has_tail = tc < ncols - nfull * TC;
@@ -252,8 +226,8 @@ __device__ __forceinline__ int smem_lupp(double *M, int n, int RS, int t, int ti
 // ---------------------------------------------------------------------------
 // Element-walk elimination with the trailing update of two steps per pass.
 //
-// Same result as smem_lupp<T, SOLVE, true> bit for bit (every element still
-// receives fma(-l_ik, u_kj, a_ij) in increasing k with the same operands).
+// Same result as smem_lupp bit for bit (every element still receives
+// fma(-l_ik, u_kj, a_ij) in increasing k with the same operands).
 // Bound by the FP64 pipe (64 clocks of a sub-partition per warp instruction,
 // full or not) and, in between, by the latency of each step's serial part:
 // the pivot search, the reciprocal, the interchange and the multipliers took
@@ -834,7 +808,7 @@ __global__ void __launch_bounds__(128) k_smem_group(SolveArgs args, int n)
             }
         }
         bad = group_any_int<T>(badv) != 0;
-        info = smem_lupp<T, MODE == kGesv, false>(M, n, RS, t, args.tile, args.threshold);
+        info = smem_lupp<T, MODE == kGesv>(M, n, RS, t, args.tile, args.threshold);
     }
     if (bad) info = -1;
 
@@ -880,8 +854,8 @@ __global__ void __launch_bounds__(128) k_smem_group(SolveArgs args, int n)
 
 // Ragged batches (tl_lupp_solve_batched): persistent over the bucket of
 // systems of size n (run-time), SB = blockDim/T systems per block and trip;
-// each system at its own offsets in per-system column-major storage.  Same
-// elimination as k_smem_group (smem_lupp), binary64.
+// each system at its own offsets in per-system column-major storage.
+// Binary64, element walk (smem_lupp2).
 template <int T>
 __global__ void __launch_bounds__(128) k_smem_ragged(RaggedArgs r, int n)
 {
