@@ -108,6 +108,7 @@ __global__ void __launch_bounds__(128) k_getrs_rhs(SolveArgs args, int n, int SB
     const int q = LAYOUT == kInterleaved ? tid % SB : tid / args.nrhs;
     const int r = LAYOUT == kInterleaved ? tid / SB : tid - q * args.nrhs;
     if (q >= live || r >= args.nrhs) return;
+    const int ylim = (n - 1) * nth + 1;  // doubles from Y[0] to this thread's last entry
     const double *M = smem + q * per;
     const double *rcp = M + n * RS;
     const int *row = reinterpret_cast<const int *>(rcp + n) + n;
@@ -117,22 +118,22 @@ __global__ void __launch_bounds__(128) k_getrs_rhs(SolveArgs args, int n, int SB
                                                  : (s * args.nrhs + r) * static_cast<int64_t>(n));
     // forward: y_i = b_row(i) - sum_{j < i} l_ij y_j
     for (int i = 0; i < n; ++i) {
-        double v = B[row[i] * es];
-        const double *Mi = M + i * RS;
+        double v = B[TL_SM(row, i, n) * es];
+        const int ri = i * RS;
 #pragma unroll 4
-        for (int j = 0; j < i; ++j) v = __fma_rn(Mi[j], Y[j * nth], v);
-        Y[i * nth] = dev::neg(v);
+        for (int j = 0; j < i; ++j) v = __fma_rn(TL_SM(M, ri + j, per), TL_SM(Y, j * nth, ylim), v);
+        TL_SM(Y, i * nth, ylim) = dev::neg(v);
     }
     // back: x_i = (y_i - sum_{j > i} u_ij x_j) * RN(1/u_ii), a quotient when a
     // pivot of the system is below DBL_MIN
     const bool tiny = flags[q] != 0;
     for (int i = n - 1; i >= 0; --i) {
-        double v = dev::neg(Y[i * nth]);
-        const double *Mi = M + i * RS;
+        double v = dev::neg(TL_SM(Y, i * nth, ylim));
+        const int ri = i * RS;
 #pragma unroll 4
-        for (int j = n - 1; j > i; --j) v = __fma_rn(Mi[j], Y[j * nth], v);
-        v = tiny ? __ddiv_rn(v, Mi[i]) : __dmul_rn(v, rcp[i]);
-        Y[i * nth] = dev::neg(v);
+        for (int j = n - 1; j > i; --j) v = __fma_rn(TL_SM(M, ri + j, per), TL_SM(Y, j * nth, ylim), v);
+        v = tiny ? __ddiv_rn(v, TL_SM(M, ri + i, per)) : __dmul_rn(v, TL_SM(rcp, i, n));
+        TL_SM(Y, i * nth, ylim) = dev::neg(v);
         B[i * es] = v;
     }
 }
@@ -165,8 +166,8 @@ __global__ void __launch_bounds__(128) k_getrs_rows(SolveArgs args, int n, int)
 #pragma unroll
         for (int c = 0; c < KM; ++c) {
             const int i = t + c * T;
-            y[c] = active && i < n ? B[row[i] * es] : 0.0;
-            l[c] = i < n ? M[i * RS] : 0.0;
+            y[c] = active && i < n ? B[TL_SM(row, i, n) * es] : 0.0;
+            l[c] = i < n ? TL_SM(M, i * RS, per) : 0.0;
         }
         // forward, column by column (the next column loaded ahead)
 #pragma unroll 1
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(128) k_getrs_rows(SolveArgs args, int n, int)
 #pragma unroll
             for (int c = 0; c < KM; ++c) {
                 const int i = t + c * T;
-                ln[c] = i < n ? M[i * RS + k + 1] : 0.0;
+                ln[c] = i < n ? TL_SM(M, i * RS + k + 1, per) : 0.0;
             }
 #pragma unroll
             for (int c = KM - 1; c >= 0; --c) {
@@ -192,7 +193,7 @@ __global__ void __launch_bounds__(128) k_getrs_rows(SolveArgs args, int n, int)
             for (int c = 0; c < KM; ++c) l[c] = ln[c];
         }
         // back, column by column (l holds column n - 1)
-        double rc = rcp[n - 1];
+        double rc = TL_SM(rcp, n - 1, n);
 #pragma unroll 1
         for (int i = n - 1; i >= 0; --i) {
             const int owner = i % T, slot = i / T;
@@ -201,14 +202,14 @@ __global__ void __launch_bounds__(128) k_getrs_rows(SolveArgs args, int n, int)
             for (int c = 1; c < KM; ++c) yi = dev::sel(c == slot, y[c], yi);
             double xi;
             if (!any_tiny) xi = __dmul_rn(yi, rc);
-            else xi = tiny ? __ddiv_rn(yi, M[i * RS + i]) : __dmul_rn(yi, rc);
+            else xi = tiny ? __ddiv_rn(yi, TL_SM(M, i * RS + i, per)) : __dmul_rn(yi, rc);
             double un[KM];
 #pragma unroll
             for (int c = 0; c < KM; ++c) {
                 const int j = t + c * T;
-                un[c] = j < i - 1 ? M[j * RS + i - 1] : 0.0;
+                un[c] = j < i - 1 ? TL_SM(M, j * RS + i - 1, per) : 0.0;
             }
-            rc = rcp[i > 0 ? i - 1 : 0];
+            rc = TL_SM(rcp, i > 0 ? i - 1 : 0, n);
             xi = __shfl_sync(0xffffffffu, xi, lane0 + owner);
 #pragma unroll
             for (int c = 0; c < KM; ++c) y[c] = dev::sel(t == owner && c == slot, xi, y[c]);

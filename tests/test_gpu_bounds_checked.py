@@ -98,6 +98,34 @@ def test_shared_memory_variants_within_bounds(tl, chk, handles, variant):
     assert violations(chk) == 0
 
 
+@pytest.mark.parametrize("n,nrhs,batch", [(8, 16, 61), (12, 6, 200), (13, 32, 5), (20, 3, 700), (27, 12, 41),
+                                          (32, 32, 9), (17, 1, 4870), (24, 2, 4871), (25, 1, 4865), (32, 2, 4873)])
+def test_getrs_within_bounds(tl, chk, handles, n, nrhs, batch):
+    """The shared-memory solves with given factors, partial blocks included."""
+    h, hc = handles
+    A, _ = inputs.uniform_systems(n, batch, 4300 + n)
+    rhs = inputs.rng(4400 + n).uniform(-1, 1, size=(batch, nrhs, n))
+    for layout in (0, 1):
+        if nrhs <= 2 and layout == 0:
+            continue  # the register kernels, which the checked library leaves out
+        ld = L.pad_ld(batch)
+        F = L.matrices_to_layout(torch.from_numpy(A).to(DEV), layout, ld)
+        B = L.multi_rhs_to_layout(torch.from_numpy(rhs).to(DEV), layout, ld)
+        piv = torch.zeros(n * (ld if layout else batch), dtype=torch.int32, device=DEV)
+        info = torch.zeros(batch, dtype=torch.int32, device=DEV)
+        tl.check("getrf", tl.tl_getrf_batched(h, n, F, layout, ld, piv, info, batch), h)
+        out = []
+        for lib, hh in ((tl.library(), h), (chk, hc)):
+            X = B.clone()
+            st = lib.tl_getrs_batched(hh, n, nrhs, F.data_ptr(), piv.data_ptr(), layout, ld, X.data_ptr(), batch,
+                                      torch.cuda.current_stream().cuda_stream)
+            assert st == 0
+            torch.cuda.synchronize()
+            out.append(X.cpu().numpy())
+        assert np.array_equal(out[0].view(np.int64), out[1].view(np.int64)), layout
+    assert violations(chk) == 0
+
+
 def test_persistent_ragged_launch_within_bounds(tl, chk, handles):
     h, hc = handles
     g = inputs.rng(4200)

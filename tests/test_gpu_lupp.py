@@ -214,34 +214,59 @@ def test_one_thread_kernels(tl, h, n, layout):
     assert np.array_equal(x_2, x_g, equal_nan=True) and np.isnan(x_g[info_o != 0]).all()
 
 
-@pytest.mark.parametrize("n,batch", [(5, 1), (6, 7296), (8, 7296), (8, 7297), (9, 2432), (10, 608), (13, 609),
-                                     (16, 2432), (16, 2433), (20, 2432), (20, 2433), (26, 4865), (32, 8192),
-                                     (32, 8193)])
-def test_small_batch_rule(tl, h, n, batch):
+# (n, side): the batch rules change the default kernel at warps per SM, so the
+# lines are given as systems per SM (plus a remainder) and follow the device.
+@pytest.mark.parametrize("n,per_sm,more", [(5, 0, 1), (6, 48, 0), (8, 48, 0), (8, 48, 1), (9, 16, 0), (10, 4, 0),
+                                           (13, 4, 1), (16, 16, 0), (16, 16, 1), (20, 16, 0), (20, 16, 1), (26, 32, 1),
+                                           (32, 54, 0), (32, 54, 1)])
+def test_small_batch_rule(tl, h, n, per_sm, more):
     """Both sides of the lines where the default kernel changes with the
-    batch (152 SMs): every output equal bit for bit to one fixed variant's."""
+    batch, with zero, subnormal, huge and non-finite systems among ordinary
+    ones: every output of every call equal bit for bit to one fixed variant's."""
+    batch = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + more
     g = torch.Generator(device=DEV)
     g.manual_seed(17 * n + batch)
+    A0 = torch.empty((batch, n, n), dtype=torch.float64, device=DEV).uniform_(-1, 1, generator=g)
+    b0 = torch.empty((batch, n), dtype=torch.float64, device=DEV).uniform_(-1, 1, generator=g)
+    if batch > 40:
+        A0[3, :, n // 2] = 0.0
+        A0[5] = 0.0
+        A0[7, n - 1, 0] = float("nan")
+        A0[8] *= 2.0 ** -1060
+        A0[19, 0, 0] = 1e308
+        A0[21] *= 2.0 ** 1020
+        A0[batch - 2, n // 2] *= 2.0 ** -1040
+        A0[batch - 1, 0, n - 1] = float("inf")
     for layout in (0, 1):
         ld = L.pad_ld(batch)
-        rows = ld if layout else batch
-        A = torch.empty(n * n * rows, dtype=torch.float64, device=DEV).uniform_(-1, 1, generator=g)
-        b = torch.empty(n * rows, dtype=torch.float64, device=DEV).uniform_(-1, 1, generator=g)
+        A = L.matrices_to_layout(A0, layout, ld)
+        b = L.vectors_to_layout(b0, layout, ld)
         out = []
         for variant in (0, tl.variant_id(8, shared=True)):
             assert tl.tl_dispatch_set(h, n, layout, variant, 0) == tl.TL_OK
-            LU, x = torch.zeros_like(A), torch.zeros_like(b)
-            piv = torch.zeros(n * rows, dtype=torch.int32, device=DEV)
-            info = torch.zeros(batch, dtype=torch.int32, device=DEV)
-            tl.check("gesv", tl.tl_gesv_batched(h, n, A, None, b, x, piv, info, layout, ld, batch), h)
-            x2 = torch.zeros_like(b)
-            tl.check("gesv", tl.tl_gesv_batched(h, n, A, LU, b, x2, piv, info, layout, ld, batch), h)
-            F = A.clone()
-            tl.check("getrf", tl.tl_getrf_batched(h, n, F, layout, ld, piv, info, batch), h)
-            out.append([t.cpu().numpy().view(np.int32) for t in (x, x2, LU, F.reshape(-1)[:0] if layout else F, piv, info)])
+            res = []
+            for call in ("gesv", "gesv_lu", "getrf"):
+                F = torch.full_like(A, -7.0) if call != "getrf" else A.clone()
+                x = torch.full_like(b, -7.0)
+                piv = torch.full((b.numel(),), -7, dtype=torch.int32, device=DEV)
+                info = torch.full((batch,), -7, dtype=torch.int32, device=DEV)
+                if call == "getrf":
+                    st = tl.tl_getrf_batched(h, n, F, layout, ld, piv, info, batch)
+                else:
+                    LU = F if call == "gesv_lu" else None
+                    st = tl.tl_gesv_batched(h, n, A, LU, b, x, piv, info, layout, ld, batch)
+                tl.check(call, st, h)
+                res += [(call, name, t.cpu().numpy().reshape(-1)) for name, t in
+                        (("F", F), ("x", x), ("piv", piv), ("info", info))]
+            out.append(res)
         tl.tl_dispatch_set(h, n, layout, 0, 0)
-        for a, c in zip(*out):
-            assert np.array_equal(a, c), (n, batch, layout)
+        if batch > 40:
+            info = out[0][3][2]
+            assert info[3] == n // 2 + 1 and info[5] == 1 and info[7] == -1 and info[batch - 1] == -1
+        for (call, name, u), (_, _, v) in zip(*out):
+            # bit for bit; a NaN of x or of a factor that overflowed may carry another payload
+            same = u == v if u.dtype == np.int32 else (u.view(np.int64) == v.view(np.int64)) | (np.isnan(u) & np.isnan(v))
+            assert same.all(), (n, batch, layout, call, name, np.flatnonzero(~same)[:5])
 
 
 @pytest.mark.parametrize("layout", [0, 1], ids=["per_system", "interleaved"])
