@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(128) k_getrs_group(SolveArgs args)
     }
     // one pivot below DBL_MIN: quotients for every row of the system, as in
     // the other solves
-    tiny = group_any<T>(tiny);
+    if (__any_sync(0xffffffffu, tiny)) tiny = group_any<T>(tiny);
     for (int r = 0; r < args.nrhs; ++r) {
         double y[K];
 #pragma unroll
