@@ -557,8 +557,9 @@ def ragged_bench(tl, h, steps, warmup, torch, device, I, seed, batch=RAGGED_BATC
         out[name] = {"ms": med, "solves_per_s": batch / (med / 1e3), "max_backward_error_n_eps": be,
                      "max_forward_error_vs_x_true": fe,
                      "info_nonzero": int((info != 0).sum().item()),
-                     "launches": "bucketing (3) + plan + 1 persistent" if mode == tl.TL_RAGGED_PERSISTENT
-                                 else "bucketing (3) + 32 per-size"}
+                     "launches": "bucketing (3) + 32 per-size" if mode != tl.TL_RAGGED_PERSISTENT
+                                 else "bucketing (3) + 1 persistent" if not prec
+                                 else "bucketing (3) + route + 1 per refining size + plan + 1 persistent"}
         if prec:
             hist = torch.bincount((ref + 1).to(torch.int64), minlength=5).tolist()
             out[name]["refine_steps_hist"] = {"fallback": hist[0], "0": hist[1], "1": hist[2], "2": hist[3],

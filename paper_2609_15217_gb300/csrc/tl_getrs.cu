@@ -15,7 +15,10 @@ namespace {
 // 1740, but n = 32, 154,194, 2595 -> 3327; below n = 12 they tie.  Up to
 // n = 9 one thread's registers hold a system, so large batches stay there
 // (n = 6, 400,000, r = 32 801 against 1123) except per system from n = 8 on
-// (n = 8, r = 6 388 -> 294).  Few large systems with few right-hand sides
+// (n = 8, r = 6 388 -> 294) and interleaved up to 16 right-hand sides, beyond
+// which n = 9 loses at first (n = 9, 400,000, r = 6 399 -> 365, r = 16 965 ->
+// 936; 200,000, r = 17 531 against 540; n = 8 still gains: r = 16 817 -> 755,
+// 200,000, r = 32 854 against 752).  Few large systems with few right-hand sides
 // are better with 16 lanes each (n = 32, 200 systems, r = 6 73 against 82).
 bool thread_per_rhs(const tl_handle *h, int n, int nrhs, int layout, int64_t batch)
 {

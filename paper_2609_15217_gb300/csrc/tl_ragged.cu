@@ -189,8 +189,9 @@ int persist_lanes(const tl_handle *h, int n, int limit, int64_t batch)
         }
     }
     // a batch that gives each sub-partition few warps: wider groups, as in the
-    // fixed-size solves (1,500 systems of seven sizes 110 -> 79 us, 64 of every
-    // size 97 -> 58 us).  16 lanes only while all their warps are resident:
+    // fixed-size solves (on the device, with the large-batch lanes -> these:
+    // 1,500 systems of seven sizes 94 -> 61 us, 64 systems of all sizes mixed
+    // 78 -> 49 us).  16 lanes only while all their warps are resident:
     // at 4,864 systems 130 us against 120 with 8.
     if (!chosen && n > kPersistRegMaxN)
         for (int wide : {32, 16, 8, 4})
