@@ -354,12 +354,13 @@ tl_status tl_newton_integrate_cpu_driven(tl_handle *h, const tl_law *law, int64_
  * tl_autotune -- time the candidate kernels (thread-to-system mapping and
  * block size) for every n in [n_min, n_max] and the layout on the current
  * device, and keep the fastest per n in the handle's dispatch table (the
- * "best X" size-aware dispatcher, Sec. 4.1) for tl_gesv_batched and
- * tl_getrf_batched; tl_getrs_batched, which is not timed, returns to its
- * built-in choice, and the ragged solves keep their own table
- * (tl_autotune_ragged).  The timed batches are large: small batches keep the
- * wider groups of the built-in default (a variant set with tl_dispatch_set
- * holds for every batch).  table_path nullable: if given, the table is
+ * "best X" size-aware dispatcher, Sec. 4.1) for tl_gesv_batched.  With
+ * LU_out, and in tl_getrf_batched, the faster of that kernel and the built-in
+ * choice runs; tl_getrs_batched, which is not timed, returns to its built-in
+ * choice, and the ragged solves keep their own table (tl_autotune_ragged).
+ * The timed batches are large: small batches keep the wider groups of the
+ * built-in default (a variant set with tl_dispatch_set holds for every
+ * batch).  table_path nullable: if given, the table of tl_gesv_batched is
  * also written there as JSON.  Allocates and frees a temporary device batch;
  * must not run during stream capture.
  */

@@ -49,10 +49,10 @@ constexpr float kRefineMargin = 0.85f;
 constexpr int kTuneReps = 5;
 
 // The choice of tl_gesv_batched / tl_getrf_batched for (n, layout).
-void set_gesv_family(tl_handle *h, int n, int layout, int variant, int block, bool tuned)
+void set_gesv_family(tl_handle *h, int n, int layout, int variant, int block)
 {
     for (int op = 0; op < kOps; ++op)
-        if (op_takes_variant(op)) h->choice[n][layout][op] = Choice{variant, block, tuned};
+        if (op_takes_variant(op)) h->choice[n][layout][op] = Choice{variant, block};
 }
 
 // For tl_getrs_batched the register kernel with the same lane count when
@@ -111,7 +111,7 @@ extern "C" tl_status tl_dispatch_set(tl_handle *h, int n, tl_layout layout, int 
     for (int i = 0; i < l.count; ++i)
         if (l.v[i].kind != kKindLatency && variant_id(l.v[i].lanes, l.v[i].kind) == variant) found = true;
     if (!found) return fail_arg(h, 4);
-    set_gesv_family(h, n, layout, variant, block, false);
+    set_gesv_family(h, n, layout, variant, block);
     set_getrs(h, n, layout, variant);
     // the ragged kernels (binary64 and mixed precision): the register kernel
     // with the same lane count, or the shared-memory kernel of the same id,
@@ -166,7 +166,7 @@ extern "C" tl_status tl_autotune(tl_handle *h, int n_min, int n_max, tl_layout l
         nv = std::max<int64_t>(nv, static_cast<int64_t>(n) * l);
         batch = std::max(batch, b);
     }
-    double *dA = nullptr, *db = nullptr, *dx = nullptr;
+    double *dA = nullptr, *dLU = nullptr, *db = nullptr, *dx = nullptr;
     int32_t *dp = nullptr, *di = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaStream_t ts = nullptr;  // a private non-blocking stream: nothing else is serialized behind the tuning
@@ -178,6 +178,7 @@ extern "C" tl_status tl_autotune(tl_handle *h, int n_min, int n_max, tl_layout l
     std::vector<Row> table;
     auto cleanup = [&]() {
         cudaFree(dA);
+        cudaFree(dLU);
         cudaFree(db);
         cudaFree(dx);
         cudaFree(dp);
@@ -189,7 +190,8 @@ extern "C" tl_status tl_autotune(tl_handle *h, int n_min, int n_max, tl_layout l
             cudaStreamDestroy(ts);
         }
     };
-    if (cudaMalloc(&dA, nA * sizeof(double)) != cudaSuccess || cudaMalloc(&db, nv * sizeof(double)) != cudaSuccess ||
+    if (cudaMalloc(&dA, nA * sizeof(double)) != cudaSuccess || cudaMalloc(&dLU, nA * sizeof(double)) != cudaSuccess ||
+        cudaMalloc(&db, nv * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&dx, nv * sizeof(double)) != cudaSuccess || cudaMalloc(&dp, nv * sizeof(int32_t)) != cudaSuccess ||
         cudaMalloc(&di, batch * sizeof(int32_t)) != cudaSuccess) {
         cudaGetLastError();
@@ -207,7 +209,27 @@ extern "C" tl_status tl_autotune(tl_handle *h, int n_min, int n_max, tl_layout l
 
     for (int n = n_min; n <= n_max && st == TL_OK; ++n) {
         const int64_t bn = batch_of(n), ld = (bn + 31) / 32 * 32;
-        SolveArgs args{dA, nullptr, db, dx, dp, di, ld, bn, 1};
+        // fastest of the timed runs of one operation
+        auto time_variant = [&](int op, const Variant *v, int block, float *out) -> tl_status {
+            SolveArgs args{dA, op == kOpGesvLU ? dLU : nullptr, db, dx, dp, di, ld, bn, 1};
+            if (op == kOpGetrf) args = SolveArgs{nullptr, dLU, nullptr, nullptr, dp, di, ld, bn, 1};
+            float best = 1e30f;
+            for (int rep = 0; rep < kTuneReps; ++rep) {
+                if (op == kOpGetrf)  // factors in place
+                    cudaMemcpyAsync(dLU, dA, static_cast<size_t>(n) * n * ld * sizeof(double), cudaMemcpyDeviceToDevice,
+                                    ts);
+                cudaEventRecord(e0, ts);
+                const tl_status s2 = launch_variant(h, v, n, block, args, ts);
+                cudaEventRecord(e1, ts);
+                if (s2 != TL_OK) return s2;
+                if (cudaEventSynchronize(e1) != cudaSuccess) return fail_cuda(h, cudaGetLastError());
+                float ms = 0.f;
+                cudaEventElapsedTime(&ms, e0, e1);
+                if (rep > 0 && ms < best) best = ms;  // first run warms up
+            }
+            *out = best;
+            return TL_OK;
+        };
         const VariantList &l = registry(n, layout, kOpGesv);
         float best_ms = 1e30f;
         int best_var = 0, best_block = 0;
@@ -218,36 +240,34 @@ extern "C" tl_status tl_autotune(tl_handle *h, int n_min, int n_max, tl_layout l
                 if (block < v->lanes) continue;
                 if (v->kind >= 1 && (block / v->lanes) * smem_sys_bytes(n, v->lanes) + 1024 > static_cast<size_t>(h->max_smem_per_block))
                     continue;
-                float ms_best = 1e30f;
-                for (int rep = 0; rep < kTuneReps; ++rep) {
-                    cudaEventRecord(e0, ts);
-                    st = launch_variant(h, v, n, block, args, ts);
-                    cudaEventRecord(e1, ts);
-                    if (st != TL_OK) break;
-                    if (cudaEventSynchronize(e1) != cudaSuccess) {
-                        st = fail_cuda(h, cudaGetLastError());
-                        break;
-                    }
-                    float ms = 0.f;
-                    cudaEventElapsedTime(&ms, e0, e1);
-                    if (rep > 0 && ms < ms_best) ms_best = ms;  // first run warms up
-                }
-                if (st != TL_OK) break;
-                if (ms_best < best_ms) {
-                    best_ms = ms_best;
+                float ms = 0.f;
+                if ((st = time_variant(kOpGesv, v, block, &ms)) != TL_OK) break;
+                if (ms < best_ms) {
+                    best_ms = ms;
                     best_var = variant_id(v->lanes, v->kind);
                     best_block = block;
                 }
             }
         }
-        if (st == TL_OK && best_var) {
-            // tl_getrs_batched was not timed: its own rule by n, nrhs, layout and
-            // batch stays (n = 27, 178,062 systems, six right-hand sides:
-            // 2272 us, the register kernel of the same lanes 3781)
-            set_gesv_family(h, n, layout, best_var, best_block, true);
-            h->choice[n][layout][kOpGetrs] = Choice{0, 0};
-            table.push_back(Row{n, best_var, best_block, best_ms});
+        if (st != TL_OK || !best_var) continue;
+        h->choice[n][layout][kOpGesv] = Choice{best_var, best_block, true};
+        // with the factors stored other lanes and blocks are faster at some n
+        // (getrf n = 25 per system: the winner of gesv 876 us, the built-in
+        // choice 795): the faster of the two
+        for (int op : {static_cast<int>(kOpGesvLU), static_cast<int>(kOpGetrf)}) {
+            const Variant *own = find_variant(n, layout, op, default_lanes(n, layout, op));
+            const Variant *won = find_variant(n, layout, op, best_var);
+            float ms_own = 0.f, ms_won = 0.f;
+            if (st == TL_OK) st = time_variant(op, own, default_block(h, own, layout, op, bn), &ms_own);
+            if (st == TL_OK) st = time_variant(op, won, best_block, &ms_won);
+            if (st == TL_OK)
+                h->choice[n][layout][op] = ms_won < ms_own ? Choice{best_var, best_block, true} : Choice{0, 0};
         }
+        // tl_getrs_batched is not timed: its own rule by n, nrhs, layout and
+        // batch stays (n = 27, 178,062 systems, six right-hand sides: 2272 us,
+        // the register kernel of the same lanes 3781)
+        h->choice[n][layout][kOpGetrs] = Choice{0, 0};
+        table.push_back(Row{n, best_var, best_block, best_ms});
     }
     cleanup();
     if (st == TL_OK && table_path) {
